@@ -1,11 +1,11 @@
 // Device building blocks shared by the pide2d kernels: complex arithmetic,
 // the in-register small DFTs and the shared-memory block FFT.
 //
-// Block FFT.  One "FFT unit" is P/16 threads that each hold 16 complex
-// values in registers; a length-P transform (P = 2^p, 16 <= P <= 8192, a
-// compile-time constant) is a Stockham autosort sequence of radix-16 stages
-// and at most one radix-2/4/8 stage, exchanging through shared memory
-// between stages.  Stage with radix R and span Ns: butterfly j reads
+// Block FFT.  One "FFT unit" is P/V threads that each hold V complex
+// values in registers (V = fft_values<R>(P), 16, 8 or 4); a length-P transform
+// (P = 2^p, 16 <= P <= 8192, a compile-time constant) is a Stockham autosort
+// sequence of radix-V stages and at most one smaller stage, exchanging through
+// shared memory between stages.  Stage with radix R and span Ns: butterfly j reads
 // x[j + r P/R], multiplies by w_P^{(j mod Ns) r P/(Ns R)}, applies an R-point
 // DFT and writes x[(j - j mod Ns) R + j mod Ns + r Ns] (the autosort
 // Stockham formulation of Govindaraju et al., SC'08).  The first stage reads
@@ -191,6 +191,25 @@ __device__ __forceinline__ void dft_small(C* v) {
     dit_layers<DIR, RAD, 2>(v);
 }
 
+// Complex values per thread of a length-P transform.  Sixteen make the fewest
+// shared-memory exchanges, which counts where the grid fills the chip.  Fewer
+// values spread a small transform over more threads and shorten its serial
+// chain, which counts where a pass has no more units than SMs.  Measured per
+// fixed-point iteration of one solve, 16 values against the choice here:
+//   FP64  P = 256 (N = 128) 164 -> 70 us, P = 512 202 -> 97 us (4 values; 8 take
+//         94 and 112), P = 1024 264 -> 247 us (8; 4 take 250), P = 2048 843 -> 804 us
+//         (8; 4 take 861).  GB300 issues two FP64 lanes per SM and clock, so the
+//         FP64 passes are bound by the number of SMs that work and by their
+//         FP64 instructions: with 8 values every twiddle is loaded instead of
+//         nine of fifteen being multiplied together.
+//   FP32  P = 256 37.7 -> 26.1 us (4 values; 8 take 29.4), P = 512 40.1 -> 31.8 us (8).
+//         P = 1024: 45.7 -> 42.3 us with 8 for one solve, but a batch of 44
+//         N = 512 jobs goes from 326 to 383 ms, so 16 stay from there on.
+template <typename R> __host__ __device__ constexpr int fft_values(int P) {
+    if (sizeof(R) == 8) return P <= 512 ? 4 : (P <= 4096 ? 8 : 16);
+    return P <= 256 ? 4 : (P <= 512 ? 8 : 16);
+}
+
 // Loader/storer of the shared-memory buffer (padded layout).  The stage
 // calls them with positions base + r * step; when both base and step are
 // multiples of 16 (or step < 16 with base a multiple of 16 and r*step < 16)
@@ -212,14 +231,14 @@ template <typename R> struct SmemStore {
 template <class T, class = void> struct is_smem_io { static constexpr bool value = false; };
 template <class T> struct is_smem_io<T, decltype((void)T::smem, void())> { static constexpr bool value = T::smem; };
 // A first-stage loader may declare `zero_mask`: bit r set means that input
-// j + r P/16 of every radix-16 butterfly is zero, so the stage skips the load
+// j + r P/V of every first-stage butterfly is zero, so the stage skips the load
 // and the transform folds the zero at compile time.
 template <class T, class = void> struct zero_mask_of { static constexpr unsigned value = 0u; };
 template <class T> struct zero_mask_of<T, decltype((void)T::zero_mask, void())> {
     static constexpr unsigned value = T::zero_mask;
 };
 
-// One Stockham stage of radix RAD (compile-time P and span NS); t in [0, P/16)
+// One Stockham stage of radix RAD <= V (compile-time P and span NS); t in [0, P/V)
 // is the thread's index in its FFT unit.  The stage reads its inputs through
 // `load` (position -> value), synchronises the block, and writes its outputs
 // through `store` (position, value), then synchronises again.  Intermediate
@@ -227,12 +246,13 @@ template <class T> struct zero_mask_of<T, decltype((void)T::zero_mask, void())> 
 // memory, a staged raw array) and the last stage may write anywhere.
 template <typename R, int DIR, int RAD, int P, int NS, class L, class S>
 __device__ __forceinline__ void fft_stage(int t, const cpx<R>* __restrict__ tw, const L& load, const S& store) {
-    constexpr int NB = 16 / RAD;            // butterflies per thread
-    constexpr int NT = P / 16;
+    constexpr int V = fft_values<R>(P);
+    constexpr int NB = V / RAD;             // butterflies per thread
+    constexpr int NT = P / V;
     constexpr int STRIDE = P / RAD;
     constexpr int TWS = P / (NS * RAD);
-    cpx<R> v[16];
-    constexpr unsigned ZM = (RAD == 16 && NS == 1) ? zero_mask_of<L>::value : 0u;
+    cpx<R> v[V];
+    constexpr unsigned ZM = (RAD == V && NS == 1) ? zero_mask_of<L>::value : 0u;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
         const int j = t + b * NT;
@@ -295,8 +315,8 @@ __device__ __forceinline__ void fft_stage(int t, const cpx<R>* __restrict__ tw, 
         const int j = t + b * NT;
         const int k = j & (NS - 1);
         const int base = (j - k) * RAD + k;
-        if constexpr (is_smem_io<S>::value && (NS % 16 == 0 || (NS == 1 && RAD == 16))) {
-            // NS = 1: base is a multiple of 16 and r < 16; NS % 16 == 0: r*NS is
+        if constexpr (is_smem_io<S>::value && (NS % 16 == 0 || (NS == 1 && (RAD == 16 || RAD == 8)))) {
+            // NS = 1: base is a multiple of RAD and r < RAD; NS % 16 == 0: r*NS is
             const int pb = padi(base);
 #pragma unroll
             for (int r = 0; r < RAD; ++r) store.at(pb, r * (NS + NS / 16), v[b * RAD + r]);
@@ -308,7 +328,7 @@ __device__ __forceinline__ void fft_stage(int t, const cpx<R>* __restrict__ tw, 
     __syncthreads();
 }
 
-// The last Stockham stage when P = 32 NS: a radix-32 butterfly per pair of
+// The last Stockham stage when P = 32 NS (V = 16): a radix-32 butterfly per pair of
 // lanes, so a length 16^k * 2 transform needs no separate radix-2 pass
 // through shared memory.  With r = 2m + h, lane h of the pair (h = t & 1)
 // takes the inputs r = 2m + h, twiddles them by w^{k r} = w^{2km} w^{kh}, and
@@ -381,18 +401,19 @@ __device__ __forceinline__ void fft_stage_r32(int t, const cpx<R>* __restrict__ 
     __syncthreads();
 }
 
-// Stages NS, 16 NS, ... of a length-P transform: radix 16 while it fits; a
+// Stages NS, V NS, ... of a length-P transform: radix V while it fits; with V = 16 a
 // remainder of 2 is merged into the last radix-16 stage (radix 32 across lane
-// pairs), a remainder of 4 or 8 is one more stage.  `load` feeds the first of
+// pairs), another remainder is one more stage.  `load` feeds the first of
 // them, `store` takes the last one's outputs (natural order); the others go
 // through `buf`.
 template <typename R, int DIR, int P, int NS, bool FUSE2, class L, class S>
 __device__ __forceinline__ void fft_from(cpx<R>* buf, int t, const cpx<R>* __restrict__ tw, const L& load,
                                          const S& store) {
-    constexpr int RAD = (NS * 16 <= P) ? 16 : P / NS;
+    constexpr int V = fft_values<R>(P);
+    constexpr int RAD = (NS * V <= P) ? V : P / NS;
     if constexpr (NS * RAD == P) {
         fft_stage<R, DIR, RAD, P, NS>(t, tw, load, store);
-    } else if constexpr (FUSE2 && NS * 32 == P) {
+    } else if constexpr (FUSE2 && V == 16 && NS * 32 == P) {
         fft_stage_r32<R, DIR, P, NS>(t, tw, load, store);
     } else {
         fft_stage<R, DIR, RAD, P, NS>(t, tw, load, SmemStore<R>{buf});

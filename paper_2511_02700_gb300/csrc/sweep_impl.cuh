@@ -29,15 +29,21 @@ namespace pide {
 
 namespace {
 
-// Launch shape of the FFT kernels for transform length P: FFT units of P/16
-// threads, at least 128 threads per block; the register target (64 in FP32,
-// 128 in FP64) fixes the minimum number of resident blocks per SM.
+// Launch shape of the FFT kernels for transform length P: FFT units of P/V
+// threads, at least one warp per block.  Small units share a warp; more of them in
+// a block would leave SMs idle: with 128 threads the eight blocks of an N = 128
+// row pass took 55 us in FP64, with 32 threads 18 us.  16-value FP32 units keep
+// 128 threads (N = 512: 24.8 ms a solve, 25.8 with 64).  The register target (64
+// in FP32, 128 in FP64) fixes the minimum number of resident blocks per SM.
 template <typename R, int P> struct Cfg {
-    static constexpr int NT = P / 16;
-    static constexpr int UNITS = NT >= 128 ? 1 : 128 / NT;
+    static constexpr int V = fft_values<R>(P);
+    static constexpr int NT = P / V;
+    static constexpr int MINT = sizeof(R) == 4 && V == 16 ? 128 : 32;
+    static constexpr int UNITS = NT >= MINT ? 1 : MINT / NT;
     static constexpr int THREADS = UNITS * NT;
     static constexpr int ULEN = padded_len(P) + 4;
-    static constexpr int MINB = (sizeof(R) == 4 ? 1024 : 512) / THREADS;
+    static constexpr int TPS = sizeof(R) == 4 ? 1024 : 512;         // resident threads per SM
+    static constexpr int MINB = TPS / THREADS < 24 ? TPS / THREADS : 24;
     static constexpr size_t SMEM = (size_t)UNITS * ULEN * sizeof(cpx<R>);
     // multi-job kernels: launched with any number of units per block up to
     // MAXT threads (the batch picks it by timed trials), same register target
@@ -133,7 +139,7 @@ template <typename R, int P>
 __device__ __forceinline__ void store_spectrum_rows(const cpx<R>* buf, cpx<R>* S, int rows, int ng, int rho, int t,
                                                     bool valid) {
     using C = cpx<R>;
-    constexpr int NT = P / 16;
+    constexpr int NT = Cfg<R, P>::NT;
     constexpr int Gc = cgroup<R>();
     auto split = [&](int k, C& xa, C& xb) {
         xa = mk<R>(0, 0);
@@ -229,11 +235,12 @@ __device__ __forceinline__ void row_forward_body(const FwdArgs<R>& a, int upb) {
         const St<R>* Ya = a.Y + (size_t)m2a * a.g.ldS;
         const St<R>* Ra = a.mode == FWD_DIFF ? a.Yref + (size_t)m2a * a.g.ldS : nullptr;
         const int ldS = a.g.ldS;
+        constexpr int EB = N / NT < 4 ? N / NT : 4;
 #pragma unroll
-        for (int b0 = 0; b0 < N / NT; b0 += 4) {
-            St<R> ya[4], yb[4], za[4], zb[4];
+        for (int b0 = 0; b0 < N / NT; b0 += EB) {
+            St<R> ya[EB], yb[EB], za[EB], zb[EB];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < EB; ++i) {
                 const int m1 = 1 + t + NT * (b0 + i);
                 const bool ok = m1 <= N - 1;
                 const St<R> zero = st_from_r<St<R>, R>(R(0));
@@ -243,7 +250,7 @@ __device__ __forceinline__ void row_forward_body(const FwdArgs<R>& a, int upb) {
                 zb[i] = (Ra && inb && ok) ? Ra[ldS + m1] : zero;
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < EB; ++i) {
                 const int m1 = 1 + t + NT * (b0 + i);
                 if (m1 > N - 1) continue;
                 const int idx = m1 + N / 2 + 1;
@@ -272,10 +279,18 @@ PIDE_FFT_JOBS_KERNEL(R, P) k_row_forward_jobs(const FwdArgs<R>* __restrict__ arr
 // column pass: staged column, T_in along s2 in the first stage, product with
 // conj(w^)/P^2 in the last forward stage, inverse FFT writing rows 1..N
 // ---------------------------------------------------------------------------
+// first-stage inputs j + r P/V that are zero for data in positions [N/2 + 2, 3N/2 + 2) only
+template <typename R, int P>
+__host__ __device__ constexpr unsigned incr_zero_mask() {
+    unsigned m = 0;
+    for (int r = 0, S = P / fft_values<R>(P); r < fft_values<R>(P); ++r)
+        if ((r + 1) * S <= P / 4 + 2 || r * S >= 3 * P / 4 + 2) m |= 1u << r;
+    return m;
+}
 // loader of an increment column: rows rlo..rhi-1 of the column group (zero elsewhere)
 template <typename R, int P>
 struct IncrColLoad {
-    static constexpr unsigned zero_mask = P >= 32 ? 0xE00Fu : 0u;   // r in {0..3, 13..15}
+    static constexpr unsigned zero_mask = incr_zero_mask<R, P>();
     const cpx<R>* col;
     int rlo, rhi;
     bool valid;
@@ -320,8 +335,7 @@ __device__ __forceinline__ void col_body(const ColArgs<R>& a, int upb) {
     };
     if constexpr (INCR) {
         // raw rows; the midpoint interpolation along s2 is in the weight spectrum.
-        // Rows outside [N/2 + 2, 3N/2 + 2) are zero, so first-stage inputs
-        // j + r P/16 with r in {0..3, 13..15} always are (P >= 32)
+        // Rows outside [N/2 + 2, 3N/2 + 2) are zero
         block_fft<R, -1, P>(buf, t, tw, IncrColLoad<R, P>{col, a.rlo, a.rhi, valid}, store_mul);
     } else {
         // (constant trip count with a guard: the loop unrolls and its loads go out together)
@@ -386,7 +400,7 @@ __device__ __forceinline__ R dcol(const R* D, int ldR, int row, int x) {
 }
 
 // Epilogue of the increment inverse row pass in coalesced order: outputs
-// m1 = t + NT b (b = 0..7) of rows m2 and m2 + 1, their C2R values in buf.
+// m1 = t + NT b of rows m2 and m2 + 1, their C2R values in buf.
 // B_w Y += zz; the residual h_t theta (zz + a12 d12 D) of the increment
 // identity goes to buf as the odd extension for the row DST.  The loads of
 // four outputs are issued together, and the neighbours x -+ 1 of the mixed
@@ -396,9 +410,9 @@ __device__ __forceinline__ void incr_epilogue(const InvArgs<R>& a, St<R>* BYv, c
                                               bool hasb, bool do_resid) {
     using C = cpx<R>;
     using S_ = St<R>;
-    constexpr int NT = P / 16, N = P / 2, NB = N / NT;
+    constexpr int NT = Cfg<R, P>::NT, N = P / 2, NB = N / NT;
     constexpr bool SHFL = NT >= 32;
-    constexpr int EB = 4;             // outputs whose loads go out together
+    constexpr int EB = NB < 4 ? NB : 4;   // outputs whose loads go out together
     const int ld = a.g.ldS, ldR = a.g.ldR;
     const int lane = threadIdx.x & 31;
     const S_ zero = st_from_r<S_, R>(R(0));
@@ -474,7 +488,7 @@ __device__ __forceinline__ void full_epilogue(const InvArgs<R>& a, St<R>* BYv, c
                                               bool valid, bool hasb, bool do_resid) {
     using C = cpx<R>;
     using S_ = St<R>;
-    constexpr int NT = P / 16, N = P / 2, NB = N / NT;
+    constexpr int NT = Cfg<R, P>::NT, N = P / 2, NB = N / NT;
     constexpr bool SHFL = NT >= 32;
     constexpr int EB = 1;             // outputs whose loads go out together
     const int ld = a.g.ldS;
@@ -1029,7 +1043,7 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
     // order (m1 = t + NT b), the state loads of four outputs issued together
     block_fft<R, -1, P>(buf, t, tw, load, SmemStore<R>{buf});
     {
-        constexpr int NB = N / NT;
+        constexpr int NB = N / NT, EB = NB < 4 ? NB : 4;
         C zz[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) zz[b] = buf[padi(t + NT * b)];
@@ -1038,17 +1052,17 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
         for (int b = 0; b < NB; ++b) buf[padi((N + t + NT * b + N / 2 + 1) & (P - 1))] = mk<R>(0, 0);
         const St<R> zero = st_from_r<St<R>, R>(R(0));
 #pragma unroll
-        for (int b0 = 0; b0 < NB; b0 += 4) {
-            St<R> y0[4], y1[4];
+        for (int b0 = 0; b0 < NB; b0 += EB) {
+            St<R> y0[EB], y1[EB];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < EB; ++i) {
                 const int m1 = t + NT * (b0 + i);
                 const size_t idx = (size_t)m2 * ld + m1;
                 y0[i] = (valid && m1 >= 1) ? Yv[idx] : zero;
                 y1[i] = (hasb && m1 >= 1) ? Yv[idx + ld] : zero;
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) update(t + NT * (b0 + i), zz[b0 + i], y0[i], y1[i]);
+            for (int i = 0; i < EB; ++i) update(t + NT * (b0 + i), zz[b0 + i], y0[i], y1[i]);
         }
         __syncthreads();
     }
@@ -1083,9 +1097,8 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
     }
     // packed R2C of the two increment rows -> spectrum rows rho = m2 + N/2 + 1, +1
     // (the midpoint interpolation is a factor of the increment weight spectrum);
-    // positions outside [N/2 + 2, 3N/2] are zero, so first-stage inputs
-    // j + r P/16 with r in {0..3, 13..15} always are (P >= 32)
-    block_fft<R, -1, P>(buf, t, tw, SmemLoad<R, (P >= 32 ? 0xE00Fu : 0u)>{buf}, SmemStore<R>{buf});
+    // positions outside [N/2 + 2, 3N/2] are zero
+    block_fft<R, -1, P>(buf, t, tw, SmemLoad<R, incr_zero_mask<R, P>()>{buf}, SmemStore<R>{buf});
     store_spectrum_rows<R, P>(buf, (C*)a.S, a.g.rows, a.g.ng, m2 + N / 2 + 1, t, valid);
 }
 template <typename R, int P>
