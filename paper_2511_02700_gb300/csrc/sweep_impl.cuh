@@ -781,20 +781,17 @@ __device__ __forceinline__ cpx<R> chunk_carry(cpx<R> v, R Qa, R Qb, cpx<R>* wsum
     return mk<R>(ea, eb);
 }
 
-// a / b: the fast FP32 quotient (2 ulp; the solve is the fixed point's
-// preconditioner, so it sets only the contraction), exact in FP64
-template <typename R> __device__ __forceinline__ R pc_div(R a, R b) {
-    if constexpr (sizeof(R) == 4) return __fdividef(a, b);
-    else return a / b;
-}
-
 // per column of the pair: th, q = e^{-th}, q^2, psi_1, q^RPT and q/c
 template <typename R> struct ColConst {
     R th, q, qq, p1, Q, g;
 };
 
-template <typename R, int P>
-__device__ __forceinline__ void col_solve_body(const ColSolveArgs<R>& a, int pair) {
+// FP32: the exponentials are cheap, and psi_{i0} is formed again in each pass that needs
+// it; the quotient is the fast one (2 ulp; the solve is the fixed point's preconditioner,
+// so it sets only the contraction)
+template <int P>
+__device__ __forceinline__ void col_solve_f32(const ColSolveArgs<float>& a, int pair) {
+    using R = float;
     using C = cpx<R>;
     using SC = ColSolveCfg<R, P>;
     constexpr int N = SC::N, RPT = SC::RPT, NW = SC::NW;
@@ -838,10 +835,10 @@ __device__ __forceinline__ void col_solve_body(const ColSolveArgs<R>& a, int pai
     const ColConst<R> ka_ = kc[0], kb_ = kc[1];
     const R q_a = ka_.q, q_b = kb_.q;
     const R Qa = ka_.Q, Qb = kb_.Q;             // q^RPT
-    // psi_i = 1 to working precision once q^{2i} < 2^-25 (FP32; 2^-54 in FP64):
+    // psi_i = 1 to working precision once q^{2i} < 2^-25:
     // then the chunk's recursions need neither psi nor the quotient
     const R thmin = ka_.th < kb_.th ? ka_.th : kb_.th;
-    const bool plain = R(2) * (R)i0 * thmin > (sizeof(R) == 4 ? R(18) : R(38));
+    const bool plain = R(2) * (R)i0 * thmin > R(18);
     // forward: z_i = psi_i b_i + q z_{i-1}
     C acc = mk<R>(R(0), R(0));
     if (plain) {
@@ -892,8 +889,8 @@ __device__ __forceinline__ void col_solve_body(const ColSolveArgs<R>& a, int pai
             const int i = i0 + r;
             const R na = pa + ea * ka_.p1, nb = pb + eb * kb_.p1;
             const bool in = i >= 1 && i <= N - 1;
-            v[r].x = in ? pc_div(ka_.g * v[r].x, pa * na) : R(0);
-            v[r].y = in ? pc_div(kb_.g * v[r].y, pb * nb) : R(0);
+            v[r].x = in ? __fdividef(ka_.g * v[r].x, pa * na) : R(0);
+            v[r].y = in ? __fdividef(kb_.g * v[r].y, pb * nb) : R(0);
             pa = na;
             pb = nb;
             ea *= ka_.qq;
@@ -943,6 +940,197 @@ __device__ __forceinline__ void col_solve_body(const ColSolveArgs<R>& a, int pai
         const int i = (int)threadIdx.x + r * SC::NTH;
         if (i >= 1 && i <= N - 1) col[(size_t)i * RS] = stage[col_pad(i)];
     }
+}
+// q^{2m} and psi_m = 1 - q^{2m} of a column: psi_{a+b} = psi_a + q^{2a} psi_b, a sum of
+// positive terms, so no value is lost to cancellation where q is near 1
+struct PsiPow {
+    double psi, e;
+};
+__device__ __forceinline__ PsiPow psi_step(PsiPow x, PsiPow y) {
+    return PsiPow{x.psi + x.e * y.psi, x.e * y.e};
+}
+
+// FP64.  The constants of a column come from one square root and one quotient,
+//     w = s/2 + sqrt(s + s^2/4),  q = 1/(1 + w),  1 - q = w q,
+// and the powers by doubling; no exponential or logarithm is evaluated, and psi_{i0} of a
+// thread's chunk is formed once and kept, psi_{i0+r} = psi_{i0} + q^{2 i0} psi_r with psi_r
+// from a table of the block.  Bound by FP64 instructions (about 20 per node) and by the
+// serial chain of the constants: 55 -> 30 us at N = 512, 27 -> 15 us at N = 128 against
+// asinh, and exp and expm1 in each pass.  (In FP32 the same form is slower: N = 4096
+// 39 -> 41 us.)
+template <int P>
+__device__ __forceinline__ void col_solve_f64(const ColSolveArgs<double>& a, int pair) {
+    using R = double;
+    using C = cpx<R>;
+    using SC = ColSolveCfg<R, P>;
+    constexpr int N = SC::N, RPT = SC::RPT, NW = SC::NW;
+    __shared__ C wsum[2][NW];
+    __shared__ C qp[17], ps[17];                // q^r and psi_r of the two columns, r <= 16
+    const int ka = 2 * pair;                    // columns ka, ka + 1 (mode k1 = column index)
+    if (ka >= N) return;                        // uniform across the block
+    constexpr int GE = rgroup<R>();
+    const int gE = ka / GE, ce = ka - gE * GE;
+    C* col = reinterpret_cast<C*>(a.E + (size_t)gE * N * GE + ce);   // row i at col[i * GE / 2]
+    constexpr int RS = GE / 2;
+    const int i0 = threadIdx.x * RPT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* stage = reinterpret_cast<C*>(smem_raw);
+    // coalesced load of the pair (rows outside 1..N-1 are zero), in flight while the first
+    // warp forms the constants
+    C v[RPT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+        const int i = (int)threadIdx.x + r * SC::NTH;
+        v[r] = (i >= 1 && i <= N - 1) ? col[(size_t)i * RS] : mk<R>(R(0), R(0));
+    }
+    const R cc = R(0.25) * a.rc2;
+    if (threadIdx.x < 32) {
+        // lane: column lane & 1, powers r = lane / 2 + 1
+        const int cl = threadIdx.x & 1, r = (threadIdx.x >> 1) + 1;
+        const R sv = (a.rc0 + a.rc1 * a.sin2[ka + cl]) / cc;
+        const R w = R(0.5) * sv + sqrt(sv + R(0.25) * sv * sv);
+        const R q = R(1) / (R(1) + w);
+        PsiPow x{R(0), R(1)}, y{w * q * (R(1) + q), q * q};
+        R pw = R(1), yw = q;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            if ((r >> j) & 1) {
+                x = psi_step(x, y);
+                pw *= yw;
+            }
+            y = PsiPow{y.psi * (R(1) + y.e), y.e * y.e};
+            yw *= yw;
+        }
+        reinterpret_cast<R*>(&qp[r])[cl] = pw;
+        reinterpret_cast<R*>(&ps[r])[cl] = x.psi;
+    }
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) stage[col_pad((int)threadIdx.x + r * SC::NTH)] = v[r];
+    __syncthreads();
+    // each thread takes its chunk of RPT consecutive rows
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) v[r] = stage[col_pad(i0 + r)];
+    const C q1 = qp[1], Q = qp[RPT];            // q, q^RPT
+    // psi and q^{2m} at the chunk's first row m = i0
+    PsiPow xa{R(0), R(1)}, xb{R(0), R(1)};
+    {
+        PsiPow ya{ps[RPT].x, Q.x * Q.x}, yb{ps[RPT].y, Q.y * Q.y};
+#pragma unroll
+        for (int j = 0; (1 << j) < SC::NTH; ++j) {
+            if ((threadIdx.x >> j) & 1) {
+                xa = psi_step(xa, ya);
+                xb = psi_step(xb, yb);
+            }
+            ya = PsiPow{ya.psi * (R(1) + ya.e), ya.e * ya.e};
+            yb = PsiPow{yb.psi * (R(1) + yb.e), yb.e * yb.e};
+        }
+    }
+    // psi_i = 1 to working precision once q^{2i} < 2^-54: then the chunk's recursions
+    // need neither psi nor the quotient
+    constexpr R kOne = 3e-17;
+    const bool plain = xa.e < kOne && xb.e < kOne;
+    // psi at row i0 + r, r >= 1 (at r = 0 the chunk's own)
+    auto psi_a = [&](int r) { return r == 0 ? xa.psi : xa.psi + xa.e * ps[r].x; };
+    auto psi_b = [&](int r) { return r == 0 ? xb.psi : xb.psi + xb.e * ps[r].y; };
+    // forward: z_i = psi_i b_i + q z_{i-1}
+    C acc = mk<R>(R(0), R(0));
+    if (plain) {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            acc.x = v[r].x + q1.x * acc.x;
+            acc.y = v[r].y + q1.y * acc.y;
+            v[r] = acc;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            acc.x = psi_a(r) * v[r].x + q1.x * acc.x;
+            acc.y = psi_b(r) * v[r].y + q1.y * acc.y;
+            v[r] = acc;
+        }
+    }
+    {
+        const C cin = chunk_carry<R, NW, false>(acc, Q.x, Q.y, wsum[0]);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            v[r].x += qp[r + 1].x * cin.x;
+            v[r].y += qp[r + 1].y * cin.y;
+        }
+    }
+    // backward: t_i = (q/c) z_i / (psi_i psi_{i+1}) + q t_{i+1}, times the row DST pair's
+    // normalisation
+    const C g = mk<R>(q1.x * a.rscale / cc, q1.y * a.rscale / cc);
+    if (plain) {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            const bool in = i0 + r <= N - 1;
+            v[r].x = in ? g.x * v[r].x : R(0);
+            v[r].y = in ? g.y * v[r].y : R(0);
+        }
+    } else if constexpr (RPT >= 4) {
+        // one quotient for four rows (1/a0 = (a1 a2 a3)/(a0 a1 a2 a3), ...); row 0's
+        // psi_0 = 0 is replaced, its value is masked
+        auto four = [&](auto psi, R gq, auto ref) {
+            R lo = i0 == 0 ? R(1) : psi(0);
+#pragma unroll
+            for (int r = 0; r < RPT; r += 4) {
+                const R p1 = psi(r + 1), p2 = psi(r + 2), p3 = psi(r + 3), p4 = psi(r + 4);
+                const R a0 = lo * p1, a1 = p1 * p2, a2 = p2 * p3, a3 = p3 * p4;
+                const R a01 = a0 * a1, a23 = a2 * a3, inv = gq / (a01 * a23);
+                const R i01 = inv * a23, i23 = inv * a01;
+                ref(r) *= i01 * a1;
+                ref(r + 1) *= i01 * a0;
+                ref(r + 2) *= i23 * a3;
+                ref(r + 3) *= i23 * a2;
+                lo = p4;
+            }
+        };
+        four(psi_a, g.x, [&](int r) -> R& { return v[r].x; });
+        four(psi_b, g.y, [&](int r) -> R& { return v[r].y; });
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (i0 + r < 1 || i0 + r > N - 1) v[r] = mk<R>(R(0), R(0));
+    } else {
+        R pa = xa.psi, pb = xb.psi;
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            const int i = i0 + r;
+            const R na = psi_a(r + 1), nb = psi_b(r + 1);
+            const bool in = i >= 1 && i <= N - 1;
+            v[r].x = in ? g.x * v[r].x / (pa * na) : R(0);
+            v[r].y = in ? g.y * v[r].y / (pb * nb) : R(0);
+            pa = na;
+            pb = nb;
+        }
+    }
+    acc = mk<R>(R(0), R(0));
+#pragma unroll
+    for (int r = RPT - 1; r >= 0; --r) {
+        acc.x = v[r].x + q1.x * acc.x;
+        acc.y = v[r].y + q1.y * acc.y;
+        v[r] = acc;
+    }
+    // x_i = psi_i t_i, staged for a coalesced store of rows 1..N-1 (the chunk reads of
+    // every thread ended before the first scan's barrier)
+    {
+        const C cin = chunk_carry<R, NW, true>(acc, Q.x, Q.y, wsum[1]);
+#pragma unroll
+        for (int r = RPT - 1; r >= 0; --r) {
+            const R ta = v[r].x + qp[RPT - r].x * cin.x, tb = v[r].y + qp[RPT - r].y * cin.y;
+            stage[col_pad(i0 + r)] = plain ? mk<R>(ta, tb) : mk<R>(psi_a(r) * ta, psi_b(r) * tb);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+        const int i = (int)threadIdx.x + r * SC::NTH;
+        if (i >= 1 && i <= N - 1) col[(size_t)i * RS] = stage[col_pad(i)];
+    }
+}
+template <typename R, int P>
+__device__ __forceinline__ void col_solve_body(const ColSolveArgs<R>& a, int pair) {
+    if constexpr (sizeof(R) == 4) col_solve_f32<P>(a, pair);
+    else col_solve_f64<P>(a, pair);
 }
 template <typename R, int P>
 __global__ void __launch_bounds__(ColSolveCfg<R, P>::NTH, ColSolveCfg<R, P>::MINB) k_col_solve(const __grid_constant__ ColSolveArgs<R> a) {
