@@ -1340,31 +1340,25 @@ PIDE_FFT_KERNEL(R, P) k_row_dst(Geometry g, const double* __restrict__ src, R* _
 
 // ---------------------------------------------------------------------------
 // per-step preparation: W = T_SL[Z] (Algorithm 1 step 2), Y^{n,0} (eq. 3.26),
-// far field on the boundary ring of Y.  Z - V at interior nodes comes from
-// k_explicit (one pass), so the SL taps read it instead of recomputing the
-// stencil per tap.
+// far field on the boundary ring of Y.  In FP32-bulk mode Z - V at interior nodes
+// comes from k_explicit (one pass), so the SL taps read it instead of recomputing
+// the stencil per tap; in FP64 one kernel does both (prep_tile_f64).
 // ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ double far_dbl(const PrepArgs<R>& a, int q1, int q2, double Kd) {
-    return (double)far_value<double>(a.payoff, Kd, a.E1d[q1 + a.g.eoff], a.E2d[q2 + a.g.eoff]);
+__device__ __forceinline__ double far_dbl(const PrepArgs<double>& a, int q1, int q2, double Kd) {
+    return far_value<double>(a.payoff, Kd, a.E1d[q1 + a.g.eoff], a.E2d[q2 + a.g.eoff]);
 }
-// the far field at node (q1, q2) as a state value: FP64 in FP64 mode, a
-// double-float pair from the split e^{s} tables in FP32-bulk mode (no FP64
-// instruction in the step's preparation); prev selects tau_{n-1}, else tau_n
-template <typename R>
-__device__ __forceinline__ St<R> far_state(const PrepArgs<R>& a, int q1, int q2, bool prev) {
-    if constexpr (sizeof(R) == 4) {
-        const int i1 = q1 + a.g.eoff, i2 = q2 + a.g.eoff;
-        return far_value_df(a.payoff, prev ? a.Kdp_h : a.Kdn_h, prev ? a.Kdp_l : a.Kdn_l, a.E1h[i1], a.E1l[i1],
-                            a.E2h[i2], a.E2l[i2]);
-    } else {
-        return far_dbl(a, q1, q2, prev ? a.Kd_prev : a.Kd_now);
-    }
+// the far field at node (q1, q2) as a state value in FP32-bulk mode: a double-float pair
+// from the split e^{s} tables (no FP64 instruction in the step's preparation); prev selects
+// tau_{n-1}, else tau_n
+__device__ __forceinline__ float2 far_state(const PrepArgs<float>& a, int q1, int q2, bool prev) {
+    const int i1 = q1 + a.g.eoff, i2 = q2 + a.g.eoff;
+    return far_value_df(a.payoff, prev ? a.Kdp_h : a.Kdn_h, prev ? a.Kdp_l : a.Kdn_l, a.E1h[i1], a.E1l[i1],
+                        a.E2h[i2], a.E2l[i2]);
 }
 
 // cz = h_t (1-theta) (D V - r_w V + B V) at interior nodes (Z - V of Algorithm 1 step 2)
-template <typename R>
-__device__ __forceinline__ void explicit_body(const PrepArgs<R>& a) {
+__device__ __forceinline__ void explicit_body(const PrepArgs<float>& a) {
+    using R = float;
     const int N = a.g.N;
     const int m1 = blockIdx.x * blockDim.x + threadIdx.x;
     const int m2 = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1376,15 +1370,14 @@ __device__ __forceinline__ void explicit_body(const PrepArgs<R>& a) {
         a.htm * (diff_state(V, idx, ld, a.d11, a.d22, a.d12) + jump_gen(a.BV[idx], V[idx], a.rw, a.rw_lo));
 }
 
-template <typename R>
-__global__ void k_explicit(const __grid_constant__ PrepArgs<R> a) { explicit_body<R>(a); }
-template <typename R>
-__global__ void k_explicit_jobs(const PrepArgs<R>* __restrict__ arr) {
-    explicit_body<R>(arr[blockIdx.z]);
+static __global__ void k_explicit(const __grid_constant__ PrepArgs<float> a) { explicit_body(a); }
+static __global__ void k_explicit_jobs(const PrepArgs<float>* __restrict__ arr) {
+    explicit_body(arr[blockIdx.z]);
 }
 
-template <typename R, int NTAP>
-__device__ __forceinline__ void prep_node(const PrepArgs<R>& a, int m1, int m2) {
+template <int NTAP>
+__device__ __forceinline__ void prep_node(const PrepArgs<float>& a, int m1, int m2) {
+    using R = float;
     const int N = a.g.N;
     if (m1 > N || m2 > N) return;
     const int ld = a.g.ldS, ldR = a.g.ldR;
@@ -1576,23 +1569,98 @@ __device__ __forceinline__ bool prep_pair_f32(const PrepArgs<float>& a, int m1, 
     return true;
 }
 
-// each thread prepares the nodes (2 tx, m2) and (2 tx + 1, m2)
-template <typename R, int NTAP>
-__device__ __forceinline__ void prep_body(const PrepArgs<R>& a) {
-    const int m1 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int m2 = blockIdx.y * blockDim.y + threadIdx.y;
-    if constexpr (sizeof(R) == 4) {
-        if (prep_pair_f32<NTAP>(a, m1, m2)) return;
+// FP64: W and Y^{n,0} of a tile of 32 x TY nodes in one pass.  Z - vref (vref: a state value
+// of the tile, so the interpolation's rounding is that of Z's variation over the tile) is
+// formed once per node of the tile and its NTAP - 1 extra rows and columns, far field outside
+// the interior, and interpolated along s1, then along s2 (the tensor weights sum to one).
+// Bound by FP64 instructions: about 16 (1 + 3/32)(1 + 3/TY) for Z, 2 NTAP for the
+// interpolation and 8 for the extrapolation, where k_explicit and one thread per node with its
+// own 16 taps took 87 and, in every warp that meets the boundary, 16 far-field evaluations
+// more (N = 128 42 -> 9.6 us, N = 512 105 -> 34 us, N = 1024 259 -> 102 us a step).  Four rows per block fill the chip at N <= 256, eight save
+// halo work above.
+template <int NTAP, int TY>
+__device__ __forceinline__ void prep_tile_f64(const PrepArgs<double>& a) {
+    constexpr int TX = 32, CX = TX + NTAP - 1, CY = TY + NTAP - 1;
+    __shared__ double dz[CY][CX + 1], hz[CY][TX];
+    const int N = a.g.N, ld = a.g.ldS;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int t = threadIdx.y * TX + threadIdx.x;
+    const double* V = a.V[0];
+    const double vref = V[(size_t)min(y0 + TY / 2, N) * ld + min(x0 + TX / 2, N)];
+    const int nx = min(TX, N + 1 - x0) + NTAP - 1, ny = min(TY, N + 1 - y0) + NTAP - 1;
+    const bool expl = a.htm != 0.0;
+    for (int i = t; i < CX * CY; i += TX * TY) {
+        const int cy = i / CX, cx = i - cy * CX;
+        if (cx >= nx || cy >= ny) continue;
+        const int q1 = x0 + a.o1 + cx, q2 = y0 + a.o2 + cy;
+        double d;
+        if (q1 >= 1 && q1 <= N - 1 && q2 >= 1 && q2 <= N - 1) {
+            const size_t idx = (size_t)q2 * ld + q1;
+            const double v = V[idx];
+            d = v - vref;
+            if (expl)
+                d += a.htm * (diff_state(V, idx, ld, a.d11, a.d22, a.d12) + jump_gen(a.BV[idx], v, a.rw, a.rw_lo));
+        } else {
+            d = far_dbl(a, q1, q2, a.Kd_prev) - vref;
+        }
+        dz[cy][cx] = d;
     }
-    prep_node<R, NTAP>(a, m1, m2);
-    prep_node<R, NTAP>(a, m1 + 1, m2);
+    __syncthreads();
+    for (int i = t; i < CY * TX; i += TX * TY) {
+        const int cy = i / TX, cx = i - cy * TX;
+        if (cx + NTAP - 1 >= nx || cy >= ny) continue;
+        double h = 0.0;
+#pragma unroll
+        for (int c = 0; c < NTAP; ++c) h += a.w1[c] * dz[cy][cx + c];
+        hz[cy][cx] = h;
+    }
+    __syncthreads();
+    const int m1 = x0 + threadIdx.x, m2 = y0 + threadIdx.y;
+    if (m1 > N || m2 > N) return;
+    const size_t idx = (size_t)m2 * ld + m1;
+    if (m1 == 0 || m2 == 0 || m1 == N || m2 == N) {
+        a.Y[idx] = far_dbl(a, m1, m2, a.Kd_now);
+        return;
+    }
+    double w = 0.0;
+#pragma unroll
+    for (int b = 0; b < NTAP; ++b) w += a.w2[b] * hz[threadIdx.y + b][threadIdx.x];
+    a.W[idx] = vref + w;
+    const double v = V[idx];
+    double e = 0.0;
+    if (a.hcount == 2) {
+        e = -(a.V[1][idx] - v);
+    } else if (a.hcount == 3) {
+        e = -3.0 * (a.V[1][idx] - v) + (a.V[2][idx] - v);
+    } else if (a.hcount >= 4) {
+        e = -6.0 * (a.V[1][idx] - v) + 4.0 * (a.V[2][idx] - v) - (a.V[3][idx] - v);
+    }
+    a.Y[idx] = v + e;
+}
+template <int NTAP, int TY>
+__global__ void __launch_bounds__(32 * TY) k_prep_tile(const __grid_constant__ PrepArgs<double> a) {
+    prep_tile_f64<NTAP, TY>(a);
+}
+template <int NTAP, int TY>
+__global__ void __launch_bounds__(32 * TY) k_prep_tile_jobs(const PrepArgs<double>* __restrict__ arr) {
+    prep_tile_f64<NTAP, TY>(arr[blockIdx.z]);
 }
 
-template <typename R, int NTAP>
-__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ PrepArgs<R> a) { prep_body<R, NTAP>(a); }
-template <typename R, int NTAP>
-__global__ void __launch_bounds__(256) k_prep_jobs(const PrepArgs<R>* __restrict__ arr) {
-    prep_body<R, NTAP>(arr[blockIdx.z]);
+// FP32-bulk: each thread prepares the nodes (2 tx, m2) and (2 tx + 1, m2)
+template <int NTAP>
+__device__ __forceinline__ void prep_body(const PrepArgs<float>& a) {
+    const int m1 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int m2 = blockIdx.y * blockDim.y + threadIdx.y;
+    if (prep_pair_f32<NTAP>(a, m1, m2)) return;
+    prep_node<NTAP>(a, m1, m2);
+    prep_node<NTAP>(a, m1 + 1, m2);
+}
+
+template <int NTAP>
+__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ PrepArgs<float> a) { prep_body<NTAP>(a); }
+template <int NTAP>
+__global__ void __launch_bounds__(256) k_prep_jobs(const PrepArgs<float>* __restrict__ arr) {
+    prep_body<NTAP>(arr[blockIdx.z]);
 }
 
 // ---------------------------------------------------------------------------
@@ -2021,19 +2089,32 @@ cudaError_t launch_dst_row_jobs(const DstRowArgs<R>& a0, const DstRowArgs<R>* ar
     PIDE_SWITCH_P(a0.g.P, CASE)
 #undef CASE
 }
+template <int TY>
+cudaError_t launch_prep_tile(const PrepArgs<double>& a, const PrepArgs<double>* arr, int K, cudaStream_t s) {
+    const dim3 blk(32, TY), grd((a.g.N + 1 + 31) / 32, (a.g.N + 1 + TY - 1) / TY, K);
+    if (arr && a.nt == 2) k_prep_tile_jobs<2, TY><<<grd, blk, 0, s>>>(arr);
+    else if (arr) k_prep_tile_jobs<4, TY><<<grd, blk, 0, s>>>(arr);
+    else if (a.nt == 2) k_prep_tile<2, TY><<<grd, blk, 0, s>>>(a);
+    else k_prep_tile<4, TY><<<grd, blk, 0, s>>>(a);
+    return cudaGetLastError();
+}
 template <typename R>
 cudaError_t launch_prep_jobs(const PrepArgs<R>& a0, const PrepArgs<R>* arr, int K, bool explicit_part, cudaStream_t s) {
-    const dim3 blk(32, 8);
-    const dim3 grd((a0.g.N + 1 + 31) / 32, (a0.g.N + 1 + 7) / 8, K);
-    if (explicit_part) {
-        k_explicit_jobs<R><<<grd, blk, 0, s>>>(arr);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    if constexpr (sizeof(R) == 8) {
+        return a0.g.N <= 256 ? launch_prep_tile<4>(a0, arr, K, s) : launch_prep_tile<8>(a0, arr, K, s);
+    } else {
+        const dim3 blk(32, 8);
+        const dim3 grd((a0.g.N + 1 + 31) / 32, (a0.g.N + 1 + 7) / 8, K);
+        if (explicit_part) {
+            k_explicit_jobs<<<grd, blk, 0, s>>>(arr);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        const dim3 grp((a0.g.N + 1 + 63) / 64, (a0.g.N + 1 + 7) / 8, K);      // two nodes per thread
+        if (a0.nt == 2) k_prep_jobs<2><<<grp, blk, 0, s>>>(arr);
+        else k_prep_jobs<4><<<grp, blk, 0, s>>>(arr);
+        return cudaGetLastError();
     }
-    const dim3 grp((a0.g.N + 1 + 63) / 64, (a0.g.N + 1 + 7) / 8, K);      // two nodes per thread
-    if (a0.nt == 2) k_prep_jobs<R, 2><<<grp, blk, 0, s>>>(arr);
-    else k_prep_jobs<R, 4><<<grp, blk, 0, s>>>(arr);
-    return cudaGetLastError();
 }
 
 template <typename R>
@@ -2096,17 +2177,21 @@ cudaError_t launch_row_dst(const Geometry& g, const double* src, R* E, const voi
 }
 template <typename R>
 cudaError_t launch_prep(const PrepArgs<R>& a, cudaStream_t s) {
-    const dim3 blk(32, 8);
-    const dim3 grd((a.g.N + 1 + 31) / 32, (a.g.N + 1 + 7) / 8);
-    const dim3 grp((a.g.N + 1 + 63) / 64, (a.g.N + 1 + 7) / 8);     // two nodes per thread
-    if (a.htm != R(0)) {
-        k_explicit<R><<<grd, blk, 0, s>>>(a);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    if constexpr (sizeof(R) == 8) {
+        return a.g.N <= 256 ? launch_prep_tile<4>(a, nullptr, 1, s) : launch_prep_tile<8>(a, nullptr, 1, s);
+    } else {
+        const dim3 blk(32, 8);
+        const dim3 grd((a.g.N + 1 + 31) / 32, (a.g.N + 1 + 7) / 8);
+        const dim3 grp((a.g.N + 1 + 63) / 64, (a.g.N + 1 + 7) / 8);     // two nodes per thread
+        if (a.htm != R(0)) {
+            k_explicit<<<grd, blk, 0, s>>>(a);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        if (a.nt == 2) k_prep<2><<<grp, blk, 0, s>>>(a);
+        else k_prep<4><<<grp, blk, 0, s>>>(a);
+        return cudaGetLastError();
     }
-    if (a.nt == 2) k_prep<R, 2><<<grp, blk, 0, s>>>(a);
-    else k_prep<R, 4><<<grp, blk, 0, s>>>(a);
-    return cudaGetLastError();
 }
 template <typename R>
 cudaError_t launch_ps_tin(int P, int nin, int nx1, const int* s, const double* w, const double* V, R* A,
