@@ -92,8 +92,8 @@ void fill_layout(int N, Layout& L) {
     L.size[R_S] = (size_t)g.ng * g.rows * cgroup_bytes<R>();
     L.size[R_WH] = L.size[R_WHI] = (size_t)g.ng * g.P * cgroup_bytes<R>();
     L.size[R_E] = (size_t)g.nge * N * rgroup_bytes<R>();
-    L.size[R_TWR] = (size_t)tw_entries(g.P) * 2 * sizeof(R);   // base table + stage tables
-    L.size[R_TWD] = (size_t)tw_entries(g.P) * 16;
+    L.size[R_TWR] = (size_t)tw_entries<R>(g.P) * 2 * sizeof(R);   // base table + stage tables
+    L.size[R_TWD] = (size_t)tw_entries<double>(g.P) * 16;
     const size_t tl = (size_t)(2 * N + 7);
     L.size[R_E1D] = L.size[R_E2D] = tl * 8;
     L.size[R_E1F] = L.size[R_E2F] = tl * 4;
@@ -2186,8 +2186,8 @@ void price_layout(pide2d_price* H) {
     H->off_params = take(16 * 8);
     H->off_rows = take((size_t)spectrum_groups<double>(P) * P * cgroup_bytes<double>());
     H->off_wh = take((size_t)ng * P * cgroup_bytes<R>());
-    H->off_twr = take((size_t)tw_entries(P) * 2 * sizeof(R));
-    H->off_twd = take((size_t)tw_entries(P) * 16);
+    H->off_twr = take((size_t)tw_entries<R>(P) * 2 * sizeof(R));
+    H->off_twd = take((size_t)tw_entries<double>(P) * 16);
     H->off_tin_s = take((size_t)H->nin * 4);
     H->off_tin_w = take((size_t)H->nin * 4 * 8);
     H->off_tout_t = take((size_t)H->nx1 * 4);

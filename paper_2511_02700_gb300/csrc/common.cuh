@@ -62,7 +62,11 @@ __host__ __device__ constexpr bool tw_has_r32(int P) {
     while (32 * s < P) s *= 16;
     return 32 * s == P;
 }
-__host__ __device__ constexpr int tw_entries(int P) { return tw32_offset(P) + (tw_has_r32(P) ? 8 * (P / 32) : 0); }
+// entries of the table: FP32 as above; FP64 holds w^k twice, as doubles and as the Q62
+// halves of the block fixed-point transform (fixfft.cuh), an int4 each
+template <typename R> __host__ __device__ constexpr int tw_entries(int P) {
+    return sizeof(R) == 8 ? 2 * P : tw32_offset(P) + (tw_has_r32(P) ? 8 * (P / 32) : 0);
+}
 
 // two adjacent table entries with one 16-byte load (two 16-byte loads in FP64)
 template <typename R>
@@ -196,12 +200,9 @@ __device__ __forceinline__ void dft_small(C* v) {
 // values spread a small transform over more threads and shorten its serial
 // chain, which counts where a pass has no more units than SMs.  Measured per
 // fixed-point iteration of one solve, 16 values against the choice here:
-//   FP64  P = 256 (N = 128) 164 -> 70 us, P = 512 202 -> 97 us (4 values; 8 take
-//         94 and 112), P = 1024 264 -> 247 us (8; 4 take 250), P = 2048 843 -> 804 us
-//         (8; 4 take 861).  GB300 issues two FP64 lanes per SM and clock, so the
-//         FP64 passes are bound by the number of SMs that work and by their
-//         FP64 instructions: with 8 values every twiddle is loaded instead of
-//         nine of fifteen being multiplied together.
+//   FP64  (with FP64 butterflies) P = 256 (N = 128) 164 -> 70 us, P = 512 202 -> 97 us
+//         (4 values; 8 take 94 and 112), P = 1024 264 -> 247 us (8; 4 take 250),
+//         P = 2048 843 -> 804 us (8; 4 take 861).
 //   FP32  P = 256 37.7 -> 26.1 us (4 values; 8 take 29.4), P = 512 40.1 -> 31.8 us (8).
 //         P = 1024: 45.7 -> 42.3 us with 8 for one solve, but a batch of 44
 //         N = 512 jobs goes from 326 to 383 ms, so 16 stay from there on.
@@ -419,18 +420,6 @@ __device__ __forceinline__ void fft_from(cpx<R>* buf, int t, const cpx<R>* __res
         fft_stage<R, DIR, RAD, P, NS>(t, tw, load, SmemStore<R>{buf});
         fft_from<R, DIR, P, NS * RAD, FUSE2>(buf, t, tw, SmemLoad<R>{buf}, store);
     }
-}
-
-// Unscaled length-P complex DFT (DIR = -1: e^{-2 pi i jk/P}, DIR = +1: e^{+...})
-// with input x[j] = load(j) and output X[k] handed to store(k, X[k]);
-// tw is the twiddle table laid out as tw_entries(P) above.  FUSE2 = false keeps a remainder of 2 as its own
-// stage (for store functors heavy enough that the radix-32 stage spills).  Every thread of the block must call it (it
-// synchronises the block); inputs read from `buf` must have been written and
-// synchronised before the call.
-template <typename R, int DIR, int P, bool FUSE2 = true, class L, class S>
-__device__ __forceinline__ void block_fft(cpx<R>* buf, int t, const cpx<R>* __restrict__ tw, const L& load,
-                                          const S& store) {
-    fft_from<R, DIR, P, 1, FUSE2>(buf, t, tw, load, store);
 }
 
 // Hint to the bulk-copy engine to bring [p, p + bytes) into L2 (no wait, no

@@ -19,6 +19,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fixfft.cuh"
 #include "internal.h"
 #include "state.cuh"
 
@@ -340,7 +341,14 @@ __global__ void k_tables(int N, double s1, double s2, double h, double* E1d, dou
 template <typename R>
 __global__ void k_twiddles(int P, cpx<R>* tw) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= tw_entries(P)) return;
+    if (i >= tw_entries<R>(P)) return;
+    if (sizeof(R) == 8 && i >= P) {          // the Q62 halves of w^{i - P}
+        double s, c;
+        sincospi(2.0 * (double)(i - P) / P, &s, &c);
+        const FxHalf re = fx_q62(c), im = fx_q62(-s);
+        reinterpret_cast<int4*>(tw)[i] = make_int4(re.h, re.l, im.h, im.l);
+        return;
+    }
     // exponent of w = e^{-2 pi i / P} held by entry i (layout in common.cuh)
     long long e = i;
     if (i >= P) {
@@ -487,7 +495,7 @@ cudaError_t launch_tables(int N, double s_lo1, double s_lo2, double h, double* E
 }
 template <typename R>
 cudaError_t launch_twiddles(int P, void* tw, cudaStream_t s) {
-    k_twiddles<R><<<(tw_entries(P) + 255) / 256, 256, 0, s>>>(P, (cpx<R>*)tw);
+    k_twiddles<R><<<(tw_entries<R>(P) + 255) / 256, 256, 0, s>>>(P, (cpx<R>*)tw);
     return cudaGetLastError();
 }
 template <typename R>

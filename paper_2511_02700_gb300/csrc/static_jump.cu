@@ -42,7 +42,7 @@ constexpr size_t kGb = cgroup_bytes<double>();
 constexpr size_t kOffWt = kOffS + al256(kNg * (kP + 2) * kGb);              // FP64 row spectra of Omega
 constexpr size_t kOffWh = kOffWt + al256(kNg * kP * kGb);                   // conj(omega-hat) / P^2
 constexpr size_t kOffTw = kOffWh + al256(kNg * kP * kGb);                   // twiddles
-constexpr size_t kOffX = kOffTw + al256((size_t)tw_entries(kP) * 16);      // U as FP64 state field
+constexpr size_t kOffX = kOffTw + al256((size_t)tw_entries<double>(kP) * 16);      // U as FP64 state field
 constexpr size_t kOffOut = kOffX + al256((size_t)(kStaticMaxN + 1) * kLd * 8);
 constexpr size_t kStaticBytes = kOffOut + al256((size_t)(kStaticMaxN + 1) * kLd * 8);
 

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "fixfft.cuh"
 #include "internal.h"
 #include "state.cuh"
 
@@ -41,7 +42,8 @@ template <typename R, int P> struct Cfg {
     static constexpr int MINT = sizeof(R) == 4 && V == 16 ? 128 : 32;
     static constexpr int UNITS = NT >= MINT ? 1 : MINT / NT;
     static constexpr int THREADS = UNITS * NT;
-    static constexpr int ULEN = padded_len(P) + 4;
+    // staged columns reach two elements past the padded length; the FP64 transform's slots follow
+    static constexpr int ULEN = padded_len(P) + (sizeof(R) == 8 ? 12 : 4);
     static constexpr int TPS = sizeof(R) == 4 ? 1024 : 512;         // resident threads per SM
     static constexpr int MINB = TPS / THREADS < 24 ? TPS / THREADS : 24;
     static constexpr size_t SMEM = (size_t)UNITS * ULEN * sizeof(cpx<R>);
