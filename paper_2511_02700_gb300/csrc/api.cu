@@ -1192,21 +1192,72 @@ static pide2d_status do_create(pide2d* H) {
     return PIDE2D_OK;
 }
 
+// whether kernels may read or write a caller's array of doubles in place: memory of the
+// current device, aligned to its elements.  Anything else (host, managed, another device)
+// is staged in R_OUT by a strided copy.  In place, the odd pitch of (N+1) doubles costs the
+// kernels little, where a strided copy each way and a conversion between pitches cost more
+// than an iteration's passes: N = 4096 FP32-bulk probe 1.62 -> 1.21 ms, N = 512 jump sum 87 -> 70 us.
+static bool direct_field(const double* p) {
+    if (((uintptr_t)p & 7) != 0) return false;
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
+// a caller's (N+1)^2 field as kernels read it: in place, or staged in R_OUT; *ld is its pitch
+static pide2d_status field_in(pide2d* H, const double* U, const double** src, int* ld) {
+    const Geometry& g = H->L.g;
+    *src = U;
+    *ld = g.N + 1;
+    if (direct_field(U)) return PIDE2D_OK;
+    double* OUT = H->at<double>(R_OUT);
+    PIDE_CUDA(cudaMemcpy2DAsync(OUT, (size_t)g.ldS * 8, U, (size_t)(g.N + 1) * 8, (size_t)(g.N + 1) * 8, g.N + 1,
+                                cudaMemcpyDefault, H->stream));
+    *src = OUT;
+    *ld = g.ldS;
+    return PIDE2D_OK;
+}
+
+// where kernels write a result field for the caller (in place or R_OUT), and, for a staged
+// one, the copy of nodes lo..N-lo of both axes that follows them
+static double* field_out(pide2d* H, double* out, int* ld) {
+    const bool direct = direct_field(out);
+    *ld = direct ? H->L.g.N + 1 : H->L.g.ldS;
+    return direct ? out : H->at<double>(R_OUT);
+}
+static pide2d_status field_out_copy(pide2d* H, double* out, const double* written, int lo) {
+    if (written == out) return PIDE2D_OK;
+    const Geometry& g = H->L.g;
+    const int N = g.N, k = N + 1 - 2 * lo;
+    PIDE_CUDA(cudaMemcpy2DAsync(out + (size_t)lo * (N + 1) + lo, (size_t)(N + 1) * 8, written + (size_t)lo * g.ldS + lo,
+                                (size_t)g.ldS * 8, (size_t)k * 8, k, cudaMemcpyDefault, H->stream));
+    return PIDE2D_OK;
+}
+
 template <typename R>
 static pide2d_status do_apply_jump(pide2d* H, const double* U, double tau, int far, double* out) {
     const Geometry g = H->L.g;
     const int N = g.N;
     cudaStream_t s = H->stream;
-    double* OUT = H->at<double>(R_OUT);
+    const double* src = nullptr;
+    int lds = 0;
+    const pide2d_status is = field_in(H, U, &src, &lds);
+    if (is != PIDE2D_OK) return is;
     St<R>* X = H->at<St<R>>(R_X);
-    PIDE_CUDA(cudaMemcpy2DAsync(OUT, (size_t)g.ldS * 8, U, (size_t)(N + 1) * 8, (size_t)(N + 1) * 8, N + 1,
-                                cudaMemcpyDefault, s));
-    PIDE_CUDA(launch_state_from_double<R>(g, OUT, g.ldS, X, s));
+    if constexpr (sizeof(R) == 4) PIDE_CUDA(launch_state_from_double<R>(g, src, lds, X, s));
     const double Kd = H->contract.strike * std::exp(-H->model.r * tau);
     FwdArgs<R> fa{};
     fa.g = g;
     fa.mode = far ? FWD_FULL : FWD_FULL0;
     fa.Y = X;
+    if constexpr (sizeof(R) == 8) {
+        fa.Y = src;
+        fa.g.ldS = lds;
+    }
     fa.E1 = (const R*)(sizeof(R) == 4 ? (const void*)H->at<float>(R_E1F) : (const void*)H->at<double>(R_E1D));
     fa.E2 = (const R*)(sizeof(R) == 4 ? (const void*)H->at<float>(R_E2F) : (const void*)H->at<double>(R_E2D));
     fa.Kd = (R)Kd;
@@ -1230,12 +1281,11 @@ static pide2d_status do_apply_jump(pide2d* H, const double* U, double tau, int f
     ia.mode = INV_OUT;
     ia.do_resid = 0;
     ia.S = H->at<void>(R_S);
-    ia.out = OUT;
+    ia.out = field_out(H, out, &ia.g.ldS);      // the field U was read before this pass
     ia.tw = H->at<void>(R_TWR);
     PIDE_CUDA(launch_row_inverse<R>(ia, s));
-    // interior block only
-    PIDE_CUDA(cudaMemcpy2DAsync(out + (N + 1) + 1, (size_t)(N + 1) * 8, OUT + g.ldS + 1, (size_t)g.ldS * 8,
-                                (size_t)(N - 1) * 8, N - 1, cudaMemcpyDefault, s));
+    const pide2d_status os = field_out_copy(H, out, ia.out, 1);   // interior block only
+    if (os != PIDE2D_OK) return os;
     PIDE_CUDA(cudaStreamSynchronize(s));
     return PIDE2D_OK;
 }
@@ -1243,7 +1293,7 @@ static pide2d_status do_apply_jump(pide2d* H, const double* U, double tau, int f
 // One iteration of the increment loop on a caller residual (pide2d_iteration_probe):
 // the DST solve of the non-mixed operator, the increment's B_w sweep and the
 // eq. 3.25 quantity, through the kernels and launch shapes of the time loop.
-// Scratch: R_OUT (the residual in FP64), R_X (Y, from zero), R_W (B_w Y, from
+// Scratch: R_OUT (staging of host fields), R_X (Y, from zero), R_W (B_w Y, from
 // zero); W is rebuilt at the start of every theta step, so a probe between
 // steps does not disturb the time loop.
 template <typename R>
@@ -1252,12 +1302,13 @@ static pide2d_status do_iteration_probe(pide2d* H, const double* r, double ht, d
     const Geometry g = H->L.g;
     const int N = g.N;
     cudaStream_t s = H->stream;
-    double* OUT = H->at<double>(R_OUT);
     St<R>* Y = H->at<St<R>>(R_X);
     St<R>* BY = H->at<St<R>>(R_W);
-    PIDE_CUDA(cudaMemcpy2DAsync(OUT, (size_t)g.ldS * 8, r, (size_t)(N + 1) * 8, (size_t)(N + 1) * 8, N + 1,
-                                cudaMemcpyDefault, s));
-    PIDE_CUDA(launch_row_dst<R>(g, OUT, H->at<R>(R_E), H->at<void>(R_TWR), s));
+    Geometry gr = g;
+    const double* src = nullptr;
+    const pide2d_status is = field_in(H, r, &src, &gr.ldS);
+    if (is != PIDE2D_OK) return is;
+    PIDE_CUDA(launch_row_dst<R>(gr, src, H->at<R>(R_E), H->at<void>(R_TWR), s));
     PIDE_CUDA(cudaMemsetAsync(Y, 0, H->L.size[R_X], s));
     PIDE_CUDA(cudaMemsetAsync(BY, 0, H->L.size[R_W], s));
     SolveSpec<R> sp{};
@@ -1281,16 +1332,14 @@ static pide2d_status do_iteration_probe(pide2d* H, const double* r, double ht, d
     A.iai.do_resid = 1;
     PIDE_CUDA(launch_row_inverse<R>(A.iai, s));
     // Y = 0 + delta exactly, B_w Y = 0 + B_w delta exactly
-    const size_t ldo = (size_t)(N + 1) * 8;
-    if (delta_out) {
-        PIDE_CUDA(launch_state_to_double<R>(g, Y, OUT, g.ldS, s));
-        PIDE_CUDA(cudaMemcpy2DAsync(delta_out + (N + 1) + 1, ldo, OUT + g.ldS + 1, (size_t)g.ldS * 8,
-                                    (size_t)(N - 1) * 8, N - 1, cudaMemcpyDefault, s));
-    }
-    if (bdelta_out) {
-        PIDE_CUDA(launch_state_to_double<R>(g, BY, OUT, g.ldS, s));
-        PIDE_CUDA(cudaMemcpy2DAsync(bdelta_out + (N + 1) + 1, ldo, OUT + g.ldS + 1, (size_t)g.ldS * 8,
-                                    (size_t)(N - 1) * 8, N - 1, cudaMemcpyDefault, s));
+    for (int k = 0; k < 2; ++k) {
+        double* out = k == 0 ? delta_out : bdelta_out;
+        if (!out) continue;
+        int ld = 0;
+        double* dst = field_out(H, out, &ld);
+        PIDE_CUDA(launch_state_to_double<R>(g, k == 0 ? Y : BY, dst, ld, 1, s));
+        const pide2d_status os = field_out_copy(H, out, dst, 1);
+        if (os != PIDE2D_OK) return os;
     }
     double stop = 0.0;
     PIDE_CUDA(cudaMemcpyAsync(&stop, H->at<void>(R_RESID), 8, cudaMemcpyDeviceToHost, s));
@@ -1301,29 +1350,27 @@ static pide2d_status do_iteration_probe(pide2d* H, const double* r, double ht, d
 
 template <typename R>
 static pide2d_status do_get_values(pide2d* H, double* dst) {
-    const Geometry g = H->L.g;
-    const int N = g.N;
-    double* OUT = H->at<double>(R_OUT);
-    PIDE_CUDA(launch_state_to_double<R>(g, (const St<R>*)H->field(H->hist[0]), OUT, g.ldS, H->stream));
-    PIDE_CUDA(cudaMemcpy2DAsync(dst, (size_t)(N + 1) * 8, OUT, (size_t)g.ldS * 8, (size_t)(N + 1) * 8, N + 1,
-                                cudaMemcpyDefault, H->stream));
+    int ld = 0;
+    double* out = field_out(H, dst, &ld);
+    PIDE_CUDA(launch_state_to_double<R>(H->L.g, (const St<R>*)H->field(H->hist[0]), out, ld, 0, H->stream));
+    const pide2d_status os = field_out_copy(H, dst, out, 0);
+    if (os != PIDE2D_OK) return os;
     PIDE_CUDA(cudaStreamSynchronize(H->stream));
     return PIDE2D_OK;
 }
 
 template <typename R>
 static pide2d_status do_greeks(pide2d* H, double* const* outs) {
-    const Geometry g = H->L.g;
-    const int N = g.N;
-    double* OUT = H->at<double>(R_OUT);
     for (int k = 0; k < 5; ++k) {
         if (!outs[k]) continue;
-        PIDE_CUDA(launch_greeks<R>(g, (const St<R>*)H->field(H->hist[0]), H->at<double>(R_E1D),
-                                   H->at<double>(R_E2D), H->h, k, OUT, g.ldS, H->stream));
-        PIDE_CUDA(cudaMemcpy2DAsync(outs[k] + (N + 1) + 1, (size_t)(N + 1) * 8, OUT + g.ldS + 1, (size_t)g.ldS * 8,
-                                    (size_t)(N - 1) * 8, N - 1, cudaMemcpyDefault, H->stream));
-        PIDE_CUDA(cudaStreamSynchronize(H->stream));
+        int ld = 0;
+        double* out = field_out(H, outs[k], &ld);
+        PIDE_CUDA(launch_greeks<R>(H->L.g, (const St<R>*)H->field(H->hist[0]), H->at<double>(R_E1D),
+                                   H->at<double>(R_E2D), H->h, k, out, ld, H->stream));
+        const pide2d_status os = field_out_copy(H, outs[k], out, 1);
+        if (os != PIDE2D_OK) return os;
     }
+    PIDE_CUDA(cudaStreamSynchronize(H->stream));
     return PIDE2D_OK;
 }
 

@@ -239,8 +239,9 @@ template <typename R> cudaError_t launch_state_from_double(const Geometry& g, co
 template <typename R> cudaError_t launch_greeks(const Geometry& g, const St<R>* V, const double* E1d,
                                                 const double* E2d, double h, int which, double* out, int ldo,
                                                 cudaStream_t s);
+// nodes lo..N-lo of both axes
 template <typename R> cudaError_t launch_state_to_double(const Geometry& g, const St<R>* src, double* dst,
-                                                        int ld_dst, cudaStream_t s);
+                                                        int ld_dst, int lo, cudaStream_t s);
 
 // device-side fixed-point loop control (loop_ctl.cu)
 struct FpCtl {

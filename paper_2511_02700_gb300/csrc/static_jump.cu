@@ -135,14 +135,17 @@ extern "C" pide2d_status pide2d_jump_static(int n, const double* omega, const do
     PIDE_STATIC_CUDA(launch_row_forward<double>(wa, s));
     PIDE_STATIC_CUDA(launch_weights_col<double>(gd, Wt, Wh, nullptr, tw, s));
 
-    // U -> state field, then one zero-padded correlation sweep
-    PIDE_STATIC_CUDA(cudaMemcpy2DAsync(OUT, (size_t)g.ldS * 8, U, (size_t)(n + 1) * 8, (size_t)(n + 1) * 8, n + 1,
-                                       cudaMemcpyDeviceToDevice, s));
-    PIDE_STATIC_CUDA(launch_state_from_double<double>(g, OUT, g.ldS, X, s));
+    // one zero-padded correlation sweep of U, read in place (staged when it is not aligned
+    // to its elements)
+    const bool in_place = ((uintptr_t)U & 7) == 0, out_place = ((uintptr_t)out & 7) == 0;
+    if (!in_place)
+        PIDE_STATIC_CUDA(cudaMemcpy2DAsync(X, (size_t)g.ldS * 8, U, (size_t)(n + 1) * 8, (size_t)(n + 1) * 8, n + 1,
+                                           cudaMemcpyDeviceToDevice, s));
     FwdArgs<double> fa{};
     fa.g = g;
     fa.mode = FWD_FULL0;
-    fa.Y = X;
+    fa.Y = in_place ? U : X;
+    if (in_place) fa.g.ldS = n + 1;
     fa.S = S;
     fa.pair0 = 0;
     fa.npairs = n + 1;
@@ -162,10 +165,12 @@ extern "C" pide2d_status pide2d_jump_static(int n, const double* omega, const do
     ia.mode = INV_OUT;
     ia.do_resid = 0;
     ia.S = S;
-    ia.out = OUT;
+    ia.out = out_place ? out : OUT;
+    if (out_place) ia.g.ldS = n + 1;
     ia.tw = tw;
     PIDE_STATIC_CUDA(launch_row_inverse<double>(ia, s));
-    PIDE_STATIC_CUDA(cudaMemcpy2DAsync(out + (n + 1) + 1, (size_t)(n + 1) * 8, OUT + g.ldS + 1, (size_t)g.ldS * 8,
-                                       (size_t)(n - 1) * 8, n - 1, cudaMemcpyDeviceToDevice, s));
+    if (!out_place)
+        PIDE_STATIC_CUDA(cudaMemcpy2DAsync(out + (n + 1) + 1, (size_t)(n + 1) * 8, OUT + g.ldS + 1, (size_t)g.ldS * 8,
+                                           (size_t)(n - 1) * 8, n - 1, cudaMemcpyDeviceToDevice, s));
     return PIDE2D_OK;
 }

@@ -31,7 +31,7 @@ namespace pide {
                                                      cudaStream_t);                                 \
     template cudaError_t launch_greeks<R>(const Geometry&, const St<R>*, const double*, const double*, \
                                           double, int, double*, int, cudaStream_t);                 \
-    template cudaError_t launch_state_to_double<R>(const Geometry&, const St<R>*, double*, int,    \
+    template cudaError_t launch_state_to_double<R>(const Geometry&, const St<R>*, double*, int, int, \
                                                    cudaStream_t);
 PIDE_INSTANTIATE(PIDE_PREC)
 #undef PIDE_INSTANTIATE

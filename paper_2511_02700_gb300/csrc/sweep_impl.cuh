@@ -1984,9 +1984,9 @@ __global__ void k_state_from_double(Geometry g, const double* src, int lds, St<R
     dst[(size_t)m2 * g.ldS + m1] = st_make<St<R>>(src[(size_t)m2 * lds + m1]);
 }
 template <typename R>
-__global__ void k_state_to_double(Geometry g, const St<R>* src, double* dst, int ldd) {
+__global__ void k_state_to_double(Geometry g, const St<R>* src, double* dst, int ldd, int lo) {
     const int m1 = blockIdx.x * blockDim.x + threadIdx.x, m2 = blockIdx.y * blockDim.y + threadIdx.y;
-    if (m1 > g.N || m2 > g.N) return;
+    if (m1 < lo || m2 < lo || m1 > g.N - lo || m2 > g.N - lo) return;
     dst[(size_t)m2 * ldd + m1] = st_dbl(src[(size_t)m2 * g.ldS + m1]);
 }
 
@@ -2307,9 +2307,9 @@ cudaError_t launch_state_from_double(const Geometry& g, const double* src, int l
     return cudaGetLastError();
 }
 template <typename R>
-cudaError_t launch_state_to_double(const Geometry& g, const St<R>* src, double* dst, int ldd, cudaStream_t s) {
+cudaError_t launch_state_to_double(const Geometry& g, const St<R>* src, double* dst, int ldd, int lo, cudaStream_t s) {
     const dim3 blk(32, 8), grd((g.N + 1 + 31) / 32, (g.N + 1 + 7) / 8);
-    k_state_to_double<R><<<grd, blk, 0, s>>>(g, src, dst, ldd);
+    k_state_to_double<R><<<grd, blk, 0, s>>>(g, src, dst, ldd, lo);
     return cudaGetLastError();
 }
 
