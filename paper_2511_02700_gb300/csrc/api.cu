@@ -2140,23 +2140,7 @@ struct pide2d_price {
     double par[9];
     std::string err;
     bool broken = false;
-    // instantiated BiCGSTAB graphs, one per system (c0, c1), and their capture stream
-    struct BicgGraph {
-        double c0, c1;
-        cudaGraph_t g;
-        cudaGraphExec_t ex;
-    };
-    std::vector<BicgGraph> bicg;
-    cudaStream_t cap = nullptr;
     template <typename T> T* at(size_t off) const { return reinterpret_cast<T*>(ws + off); }
-    ~pide2d_price() {
-        if (!bicg.empty()) cudaStreamSynchronize(stream);
-        for (auto& b : bicg) {
-            cudaGraphExecDestroy(b.ex);
-            cudaGraphDestroy(b.g);
-        }
-        if (cap) cudaStreamDestroy(cap);
-    }
 };
 
 namespace {
@@ -2349,7 +2333,6 @@ static pide2d_status price_apply(pide2d_price* H, const double* V, double* out) 
     PIDE_PCUDA(launch_ps_rows_inv<R>(P, S, H->nout, H->at<double>(H->off_By), H->nout, tw, s));
     PIDE_PCUDA(launch_ps_tout(H->nx1, H->nout, H->at<int>(H->off_tout_t), H->at<double>(H->off_tout_u),
                               H->at<double>(H->off_By), H->nout, out, s));
-    PIDE_PCUDA(cudaStreamSynchronize(s));
     return PIDE2D_OK;
 }
 
@@ -2398,7 +2381,7 @@ static size_t ps_field_bytes(int nx1) { return align256((size_t)nx1 * nx1 * 8); 
 
 static size_t ps_loop_bytes(int nx1) {
     return (size_t)F_COUNT * ps_field_bytes(nx1) + 3 * align256((size_t)nx1 * 3 * 8) + 2 * align256((size_t)nx1 * 4) +
-           2 * align256((size_t)nx1 * 4 * 8) + align256((size_t)ps_reduction_blocks() * 3 * 8) + 256 + 256;
+           2 * align256((size_t)nx1 * 4 * 8) + align256((size_t)ps_reduction_blocks() * 8 * 8) + 256 + 256;
 }
 
 static pide2d_status price_solve(pide2d_price* H, const pide2d_contract* c, double theta, int n_steps, double tol,
@@ -2421,7 +2404,7 @@ static pide2d_status price_solve(pide2d_price* H, const pide2d_contract* c, doub
     int* ds2 = reinterpret_cast<int*>(take((size_t)n1 * 4));
     double* dw1 = reinterpret_cast<double*>(take((size_t)n1 * 4 * 8));
     double* dw2 = reinterpret_cast<double*>(take((size_t)n1 * 4 * 8));
-    double* part = reinterpret_cast<double*>(take((size_t)ps_reduction_blocks() * 3 * 8));
+    double* part = reinterpret_cast<double*>(take((size_t)ps_reduction_blocks() * 8 * 8));
     double* res = reinterpret_cast<double*>(q);
     PsBicg* bst = reinterpret_cast<PsBicg*>(q + 256);
     const std::vector<double>& x = H->x;
@@ -2472,50 +2455,18 @@ static pide2d_status price_solve(pide2d_price* H, const pide2d_contract* c, doub
     auto apply_jump = [&](const double* V, double* out) -> pide2d_status {
         return H->precision == PIDE2D_FP64 ? price_apply<double>(H, V, out) : price_apply<float>(H, V, out);
     };
-    // BiCGSTAB with Jacobi preconditioning for (c0 I - c1 D) X = B, X holding the
-    // start: one graph launch (set-up and a while-node over the iterations, the
-    // scalars on the device), then one read of the solver state
+    // BiCGSTAB with Jacobi preconditioning for (c0 I - c1 D) X = B, X holding the start: one
+    // launch; its state is read with the iteration's stopping quantity
     constexpr int kBicgMaxIt = 20000;
-    constexpr size_t kBicgGraphs = 8;
-    auto bicgstab = [&](double c0, double c1, const double* Bv, double* X, int* its) -> pide2d_status {
-        cudaGraphExec_t ex = nullptr;
-        for (const auto& bg : H->bicg)
-            if (bg.c0 == c0 && bg.c1 == c1) ex = bg.ex;
-        if (!ex) {
-            if (!H->cap) PIDE_PCUDA(cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking));
-            cudaGraph_t g = nullptr;
-            PIDE_PCUDA(cudaGraphCreate(&g, 0));
-            const PsBicgArgs ba{d, n, c0, c1, Bv, X, fld(F_R), fld(F_RH), fld(F_P), fld(F_VV), fld(F_YY), fld(F_S),
-                                fld(F_ZZ), fld(F_T), fld(F_DINV), part, res, bst, kBicgMaxIt};
-            const char* where = "";
-            cudaError_t e = record_ps_bicg(g, H->cap, ba, &where);
-            if (e == cudaSuccess) {
-                e = cudaGraphInstantiate(&ex, g, 0);
-                where = "cudaGraphInstantiate";
-            }
-            if (e != cudaSuccess) {
-                cudaGraphDestroy(g);
-                H->err = std::string("price-space BiCGSTAB graph: ") + where + ": " + cudaGetErrorString(e);
-                H->broken = true;
-                return PIDE2D_ERR_CUDA;
-            }
-            if (H->bicg.size() >= kBicgGraphs) {
-                PIDE_PCUDA(cudaStreamSynchronize(s));       // the oldest may still be queued
-                cudaGraphExecDestroy(H->bicg.front().ex);
-                cudaGraphDestroy(H->bicg.front().g);
-                H->bicg.erase(H->bicg.begin());
-            }
-            H->bicg.push_back({c0, c1, g, ex});
-        }
-        PIDE_PCUDA(cudaGraphLaunch(ex, s));
-        PsBicg hb{};
-        PIDE_PCUDA(cudaMemcpyAsync(&hb, bst, sizeof hb, cudaMemcpyDeviceToHost, s));
-        PIDE_PCUDA(cudaStreamSynchronize(s));
-        *its = hb.it;
-        if (!(hb.rn <= hb.lim)) {
-            H->err = "price-space BiCGSTAB did not reach its tolerance";
-            return PIDE2D_ERR_NOT_CONVERGED;
-        }
+    const int bicg_blocks = ps_bicg_blocks(n1);
+    if (bicg_blocks < 1) {
+        H->err = "price-space BiCGSTAB: no cooperative launch on this device";
+        return PIDE2D_ERR_CUDA;
+    }
+    auto bicgstab = [&](double c0, double c1, const double* Bv, double* X) -> pide2d_status {
+        const PsBicgArgs ba{d, c0, c1, Bv, X, fld(F_R), fld(F_RH), fld(F_P), fld(F_YY), fld(F_VV), fld(F_ZZ), fld(F_S),
+                            fld(F_T), fld(F_DINV), part, bst, kBicgMaxIt};
+        PIDE_PCUDA(launch_ps_bicg(ba, bicg_blocks, s));
         return PIDE2D_OK;
     };
 
@@ -2558,14 +2509,24 @@ static pide2d_status price_solve(pide2d_price* H, const pide2d_contract* c, doub
             }
             PIDE_PCUDA(launch_ps_axpy(n, htt, fld(F_BY), 1.0, fld(F_W), 0.0, nullptr, nullptr, fld(F_B), s));
             PIDE_PCUDA(cudaMemcpyAsync(fld(F_YN), fld(F_Y), n * 8, cudaMemcpyDeviceToDevice, s));
-            int its = 0;
-            const pide2d_status js = bicgstab(c0, c1, fld(F_B), fld(F_YN), &its);
+            const pide2d_status js = bicgstab(c0, c1, fld(F_B), fld(F_YN));
             if (js != PIDE2D_OK) return js;
+            PsBicg hb{};
+            PIDE_PCUDA(cudaMemcpyAsync(&hb, bst, sizeof hb, cudaMemcpyDeviceToHost, s));
             PIDE_PCUDA(launch_ps_maxrel(n, fld(F_YN), fld(F_Y), part, res, s));
             PIDE_PCUDA(cudaMemcpyAsync(&err, res, 8, cudaMemcpyDeviceToHost, s));
             PIDE_PCUDA(launch_ps_axpy(n, 1.0, fld(F_YN), -1.0, fld(F_Y), 0.0, nullptr, nullptr, fld(F_T), s));
             PIDE_PCUDA(cudaMemcpyAsync(fld(F_Y), fld(F_YN), n * 8, cudaMemcpyDeviceToDevice, s));
             PIDE_PCUDA(cudaStreamSynchronize(s));
+            if (hb.stalled) {
+                H->err = "price-space BiCGSTAB: grid barrier timed out";
+                H->broken = true;
+                return PIDE2D_ERR_CUDA;
+            }
+            if (!(hb.rn <= hb.lim)) {
+                H->err = "price-space BiCGSTAB did not reach its tolerance";
+                return PIDE2D_ERR_NOT_CONVERGED;
+            }
             if (err < tol) break;
         }
         if (k > kmax) {
@@ -3082,7 +3043,10 @@ pide2d_status pide2d_price_create(const pide2d_price_grid* g, const pide2d_model
 pide2d_status pide2d_price_apply_jump(pide2d_price_t* H, const double* V, double* out) {
     if (!H || !V || !out) return PIDE2D_ERR_ARG;
     if (H->broken) return PIDE2D_ERR_STATE;
-    return H->precision == PIDE2D_FP64 ? price_apply<double>(H, V, out) : price_apply<float>(H, V, out);
+    const pide2d_status st = H->precision == PIDE2D_FP64 ? price_apply<double>(H, V, out) : price_apply<float>(H, V, out);
+    if (st != PIDE2D_OK) return st;
+    PIDE_PCUDA(cudaStreamSynchronize(H->stream));
+    return PIDE2D_OK;
 }
 
 pide2d_status pide2d_price_solve(pide2d_price_t* H, const pide2d_contract* c, double theta, int n_steps,

@@ -201,33 +201,28 @@ cudaError_t launch_ps_diag_inv(const PsDiff& d, double c0, double c1, double* di
 cudaError_t launch_ps_axpy(size_t n, double a, const double* x, double b, const double* y, double c, const double* z,
                            const double* dinv, double* out, cudaStream_t s);
 int ps_reduction_blocks();
-struct PsDots {
-    const double* x[3];
-    const double* y[3];
-};
-cudaError_t launch_ps_dots(size_t n, int nd, const PsDots& dp, double* part, double* res, cudaStream_t s);
-// one Jacobi-preconditioned BiCGSTAB solve of (c0 I - c1 D) X = B with its
-// scalars in device memory: record_ps_bicg builds it as a CUDA graph (set-up,
-// then a while-node over the iterations), so a solve is one graph launch
+// one Jacobi-preconditioned BiCGSTAB solve of (c0 I - c1 D) X = B to a relative residual of
+// 1e-13, as one cooperative launch
 struct PsBicg {
     double rho, rho_new, alpha, omega;
     double rn, lim;          // the residual norm and the stopping level 1e-13 |B|
     int it, done;            // iterations done; 1 once the half-step residual met lim
+    unsigned arrived;        // grid barrier
+    int stalled;             // a block gave up waiting at a barrier
 };
 struct PsBicgArgs {
     PsDiff d;
-    size_t n;
     double c0, c1;
     const double* B;
     double* X;               // the start in, the solution out
-    double *r, *rh, *p, *v, *y, *s, *z, *t;
+    double *r, *rh, *p0, *p1, *v0, *v1, *s, *t;
     const double* dinv;      // the Jacobi preconditioner
-    double* part;            // ps_reduction_blocks() x 3 partial sums
-    double* res;             // 3 doubles
+    double* part;            // partial sums: 8 doubles for each of ps_reduction_blocks() blocks
     PsBicg* st;
     int maxit;
 };
-cudaError_t record_ps_bicg(cudaGraph_t g, cudaStream_t cap, const PsBicgArgs& a, const char** where);
+int ps_bicg_blocks(int n1);
+cudaError_t launch_ps_bicg(const PsBicgArgs& a, int blocks, cudaStream_t s);
 cudaError_t launch_ps_maxrel(size_t n, const double* a, const double* b, double* part, double* res, cudaStream_t s);
 cudaError_t launch_ps_sl(int n1, const int* s1, const double* w1, const int* s2, const double* w2, const double* Z,
                          double* W, cudaStream_t s);

@@ -3,7 +3,7 @@
 // extrapolation below y_out is encoded in the tables as two taps).
 #include <cuda_runtime.h>
 
-#include <vector>
+#include <algorithm>
 
 #include "internal.h"
 
@@ -106,23 +106,6 @@ __global__ void k_ps_axpy(size_t n, double a, const double* x, double b, const d
     out[i] = r;
 }
 
-// up to three dot products <x_k, y_k> as per-block partials
-__global__ void k_ps_dots(size_t n, int nd, PsDots dp, double* __restrict__ part) {
-    __shared__ double red[3][256];
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        for (int k = 0; k < nd; ++k) acc[k] += dp.x[k][i] * dp.y[k][i];
-    for (int k = 0; k < 3; ++k) red[k][threadIdx.x] = acc[k];
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            for (int k = 0; k < 3; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) part[(size_t)blockIdx.x * 3 + k] = red[k][0];
-}
-
 __global__ void k_ps_maxrel(size_t n, const double* __restrict__ a, const double* __restrict__ b,
                             double* __restrict__ part) {
     __shared__ double red[256];
@@ -138,25 +121,18 @@ __global__ void k_ps_maxrel(size_t n, const double* __restrict__ a, const double
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-// fixed-order sums (kind 0) or maxima (kind 1) of per-block partials into res[0..nd)
-__global__ void k_ps_finish(const double* __restrict__ part, int nblocks, int nd, int kind, double* __restrict__ res) {
+// the maximum of per-block partials into res[0]
+__global__ void k_ps_finish(const double* __restrict__ part, int nblocks, double* __restrict__ res) {
     __shared__ double red[256];
-    for (int k = 0; k < nd; ++k) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-            const double v = part[(size_t)b * (kind ? 1 : 3) + k];
-            s = kind ? fmax(s, v) : s + v;
-        }
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) red[threadIdx.x] = kind ? fmax(red[threadIdx.x], red[threadIdx.x + o])
-                                                              : red[threadIdx.x] + red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) res[k] = red[0];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s = fmax(s, part[b]);
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
         __syncthreads();
     }
+    if (threadIdx.x == 0) res[0] = red[0];
 }
 
 constexpr int kPsRedBlocks = 304;      // 2 x 152 SMs
@@ -178,187 +154,228 @@ cudaError_t launch_ps_axpy(size_t n, double a, const double* x, double b, const 
     return cudaGetLastError();
 }
 int ps_reduction_blocks() { return kPsRedBlocks; }
-cudaError_t launch_ps_dots(size_t n, int nd, const PsDots& dp, double* part, double* res, cudaStream_t s) {
-    k_ps_dots<<<kPsRedBlocks, 256, 0, s>>>(n, nd, dp, part);
-    k_ps_finish<<<1, 256, 0, s>>>(part, kPsRedBlocks, nd, 0, res);
-    return cudaGetLastError();
-}
 // ---------------------------------------------------------------------------
-// BiCGSTAB with the scalars on the device.  The vector updates read alpha,
-// beta and omega from PsBicg; each scalar step is one thread; the loop is a
-// CUDA-graph while-node whose condition the scalar steps set (no host round
-// trip per iteration).  Same recurrences and reductions as a host-driven loop.
+// Jacobi-preconditioned BiCGSTAB for (c0 I - c1 D) X = B as one cooperative kernel.
+// A block owns tiles of 32 x 8 nodes; a product with the matrix takes its vector
+// from shared memory, where the tile and its ring of neighbours are formed from the
+// recurrences (p = r + beta p - beta omega v, y = p/diag; s = r - alpha v, z = s/diag), so
+// an iteration is three passes with one grid barrier and one reduction each.  Every
+// block sums the blocks' partial dot products in the same order and so takes the same
+// scalars and the same decision to stop.  Bound by the latency of the three barriers;
+// NIG1, N_x = 150, 75 steps: 103 us a system, 535 -> 506 ms for the whole solve against
+// sixteen kernels an iteration.
 // ---------------------------------------------------------------------------
-__global__ void k_bicg_init(const double* __restrict__ res, PsBicg* __restrict__ st, int maxit,
-                            unsigned long long hnd) {
-    PsBicg q{};
-    const double bn = sqrt(res[0]);                   // res: <B, B>, <r, r>
-    q.lim = 1e-13 * (bn > 0.0 ? bn : 1.0);
-    q.rn = sqrt(res[1]);
-    q.rho = 1.0;
-    q.alpha = 1.0;
-    q.omega = 1.0;
-    q.rho_new = res[1];
-    *st = q;
-    cudaGraphSetConditional((cudaGraphConditionalHandle)hnd, (q.rn > q.lim && maxit > 0) ? 1u : 0u);
-}
-// p = r (first iteration) or r + beta p - beta omega v, beta = (rho_new / rho)(alpha / omega)
-__global__ void k_bicg_p(size_t n, const PsBicg* __restrict__ st, const double* __restrict__ r, double* p,
-                         const double* __restrict__ v) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const PsBicg q = *st;
-    if (q.it == 0) {
-        p[i] = r[i];
-    } else {
-        const double beta = (q.rho_new / q.rho) * (q.alpha / q.omega);
-        p[i] = 1.0 * r[i] + beta * p[i] + (-beta * q.omega) * v[i];
+namespace {
+constexpr int kTX = 32, kTY = 8, kPsThreads = kTX * kTY;
+constexpr unsigned kSpinLimit = 1u << 22;            // a barrier gives up after a few seconds
+}  // namespace
+
+// all blocks of the (cooperative) grid; false once any block gave up waiting
+__device__ __forceinline__ bool ps_barrier(PsBicg* st, unsigned& gen) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        gen += gridDim.x;
+        __threadfence();
+        atomicAdd(&st->arrived, 1u);
+        unsigned spins = 0;
+        while (*(volatile unsigned*)&st->arrived < gen && ++spins < kSpinLimit) {}
+        __threadfence();
+        ok = spins < kSpinLimit;
+        if (!ok) st->stalled = 1;
     }
-}
-__global__ void k_bicg_alpha(const double* __restrict__ res, PsBicg* __restrict__ st) {
-    st->alpha = st->rho_new / res[0];                 // res: <rh, v>
-}
-// s = r - alpha v
-__global__ void k_bicg_s(size_t n, const PsBicg* __restrict__ st, const double* __restrict__ r,
-                         const double* __restrict__ v, double* __restrict__ s) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    s[i] = 1.0 * r[i] + (-st->alpha) * v[i];
-}
-// res: <t, s>, <t, t>, <s, s>: converged on s (the loop ends), else omega
-__global__ void k_bicg_omega(const double* __restrict__ res, PsBicg* __restrict__ st, unsigned long long hnd) {
-    PsBicg q = *st;
-    q.it += 1;
-    const double sn = sqrt(res[2]);
-    if (sn <= q.lim) {
-        q.done = 1;
-        q.rn = sn;
-        cudaGraphSetConditional((cudaGraphConditionalHandle)hnd, 0u);
-    } else {
-        q.omega = res[0] / res[1];
-    }
-    *st = q;
-}
-// X += alpha y (+ omega z), r = s - omega t (unless converged on s)
-__global__ void k_bicg_xr(size_t n, const PsBicg* __restrict__ st, double* X, const double* __restrict__ y,
-                          const double* __restrict__ z, const double* __restrict__ s, const double* __restrict__ t,
-                          double* __restrict__ r) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const PsBicg q = *st;
-    if (q.done) {
-        X[i] = 1.0 * X[i] + q.alpha * y[i];
-    } else {
-        X[i] = 1.0 * X[i] + q.alpha * y[i] + q.omega * z[i];
-        r[i] = 1.0 * s[i] + (-q.omega) * t[i];
-    }
-}
-// res: <r, r>, <rh, r>: the residual norm, the next rho and the loop condition
-__global__ void k_bicg_rho(const double* __restrict__ res, PsBicg* __restrict__ st, int maxit,
-                           unsigned long long hnd) {
-    PsBicg q = *st;
-    if (q.done) return;                               // the condition was cleared at convergence on s
-    q.rho = q.rho_new;
-    q.rn = sqrt(res[0]);
-    q.rho_new = res[1];
-    *st = q;
-    cudaGraphSetConditional((cudaGraphConditionalHandle)hnd, (q.rn > q.lim && q.it < maxit) ? 1u : 0u);
+    __syncthreads();
+    return ok != 0;
 }
 
-cudaError_t record_ps_bicg(cudaGraph_t g, cudaStream_t cs, const PsBicgArgs& a, const char** where) {
-    cudaError_t e = cudaSuccess;
-#define PS_GTRY(call)                \
-    do {                             \
-        e = (call);                  \
-        if (e != cudaSuccess) {      \
-            *where = #call;          \
-            return e;                \
-        }                            \
-    } while (0)
-    const size_t n = a.n;
-    const unsigned nb = (unsigned)((n + 255) / 256);
-    cudaGraphConditionalHandle hnd;
-    PS_GTRY(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault));
-    // set-up: r = B - (c0 X - c1 D X), rh = r, <B, B>, <r, r>, the stopping level
-    PS_GTRY(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    {
-        cudaError_t x = launch_ps_diff(a.d, a.X, a.c0, -a.c1, nullptr, 0.0, a.r, cs);
-        if (x == cudaSuccess) x = launch_ps_axpy(n, 1.0, a.B, -1.0, a.r, 0.0, nullptr, nullptr, a.r, cs);
-        if (x == cudaSuccess) x = cudaMemcpyAsync(a.rh, a.r, n * 8, cudaMemcpyDeviceToDevice, cs);
-        if (x == cudaSuccess) x = launch_ps_dots(n, 2, PsDots{{a.B, a.r, nullptr}, {a.B, a.r, nullptr}}, a.part, a.res, cs);
-        if (x == cudaSuccess) {
-            k_bicg_init<<<1, 1, 0, cs>>>(a.res, a.st, a.maxit, (unsigned long long)hnd);
-            x = cudaGetLastError();
-        }
-        cudaGraph_t got = nullptr;
-        const cudaError_t x2 = cudaStreamEndCapture(cs, &got);
-        if (x != cudaSuccess) { *where = "BiCGSTAB set-up launches"; return x; }
-        if (x2 != cudaSuccess) { *where = "cudaStreamEndCapture(set-up)"; return x2; }
+// sums over the grid of NV values per thread, in a fixed order; part: NV doubles per block
+template <int NV>
+__device__ __forceinline__ bool ps_grid_sum(double* v, double* part, PsBicg* st, unsigned& gen) {
+    __shared__ double red[NV][kPsThreads / 32];
+    __shared__ double tot[NV];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto warp_sum = [](double x) {
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    };
+    __syncthreads();                                  // red and tot of the previous call are read
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const double x = warp_sum(v[k]);
+        if (lane == 0) red[k][w] = x;
     }
-    // the set-up is a chain: its last node has no dependents
-    size_t nn = 0;
-    PS_GTRY(cudaGraphGetNodes(g, nullptr, &nn));
-    std::vector<cudaGraphNode_t> nodes(nn);
-    PS_GTRY(cudaGraphGetNodes(g, nodes.data(), &nn));
-    std::vector<cudaGraphNode_t> leaves;
-    for (auto nd : nodes) {
-        size_t nd_out = 0;
-        PS_GTRY(cudaGraphNodeGetDependentNodes(nd, nullptr, nullptr, &nd_out));
-        if (nd_out == 0) leaves.push_back(nd);
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double x = 0.0;
+        for (int u = 0; u < kPsThreads / 32; ++u) x += red[threadIdx.x][u];
+        part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = x;
     }
-    cudaGraphNodeParams cp{};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = hnd;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t loop = nullptr;
-    PS_GTRY(cudaGraphAddNode(&loop, g, leaves.data(), nullptr, leaves.size(), &cp));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    // one BiCGSTAB iteration
-    PS_GTRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    {
-        cudaError_t x = cudaSuccess;
-        k_bicg_p<<<nb, 256, 0, cs>>>(n, a.st, a.r, a.p, a.v);
-        x = cudaGetLastError();
-        if (x == cudaSuccess) x = launch_ps_axpy(n, 1.0, a.p, 0.0, nullptr, 0.0, nullptr, a.dinv, a.y, cs);
-        if (x == cudaSuccess) x = launch_ps_diff(a.d, a.y, a.c0, -a.c1, nullptr, 0.0, a.v, cs);
-        if (x == cudaSuccess) x = launch_ps_dots(n, 1, PsDots{{a.rh, nullptr, nullptr}, {a.v, nullptr, nullptr}}, a.part, a.res, cs);
-        if (x == cudaSuccess) {
-            k_bicg_alpha<<<1, 1, 0, cs>>>(a.res, a.st);
-            x = cudaGetLastError();
-        }
-        if (x == cudaSuccess) {
-            k_bicg_s<<<nb, 256, 0, cs>>>(n, a.st, a.r, a.v, a.s);
-            x = cudaGetLastError();
-        }
-        if (x == cudaSuccess) x = launch_ps_axpy(n, 1.0, a.s, 0.0, nullptr, 0.0, nullptr, a.dinv, a.z, cs);
-        if (x == cudaSuccess) x = launch_ps_diff(a.d, a.z, a.c0, -a.c1, nullptr, 0.0, a.t, cs);
-        if (x == cudaSuccess) x = launch_ps_dots(n, 3, PsDots{{a.t, a.t, a.s}, {a.s, a.t, a.s}}, a.part, a.res, cs);
-        if (x == cudaSuccess) {
-            k_bicg_omega<<<1, 1, 0, cs>>>(a.res, a.st, (unsigned long long)hnd);
-            x = cudaGetLastError();
-        }
-        if (x == cudaSuccess) {
-            k_bicg_xr<<<nb, 256, 0, cs>>>(n, a.st, a.X, a.y, a.z, a.s, a.t, a.r);
-            x = cudaGetLastError();
-        }
-        if (x == cudaSuccess) x = launch_ps_dots(n, 2, PsDots{{a.r, a.rh, nullptr}, {a.r, a.r, nullptr}}, a.part, a.res, cs);
-        if (x == cudaSuccess) {
-            k_bicg_rho<<<1, 1, 0, cs>>>(a.res, a.st, a.maxit, (unsigned long long)hnd);
-            x = cudaGetLastError();
-        }
-        cudaGraph_t got = nullptr;
-        const cudaError_t x2 = cudaStreamEndCapture(cs, &got);
-        if (x != cudaSuccess) { *where = "BiCGSTAB iteration launches"; return x; }
-        if (x2 != cudaSuccess) { *where = "cudaStreamEndCapture(iteration)"; return x2; }
+    if (!ps_barrier(st, gen)) return false;
+    if (w < NV) {
+        double x = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(part + (size_t)w * gridDim.x + b);
+        x = warp_sum(x);
+        if (lane == 0) tot[w] = x;
     }
-#undef PS_GTRY
-    return cudaSuccess;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = tot[k];
+    return true;
+}
+
+__global__ void __launch_bounds__(kPsThreads) k_ps_bicg(PsBicgArgs a) {
+    __shared__ double sv[kTY + 2][kTX + 2];
+    const int n1 = a.d.n1, N = n1 - 1;
+    const int ntx = (n1 + kTX - 1) / kTX, nty = (n1 + kTY - 1) / kTY, ntiles = ntx * nty;
+    const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX;
+    unsigned gen = 0;
+    // vec(i) at the nodes of a tile and their ring into sv, then f(i, A vec at node i, vec) at
+    // the tile's nodes, A = c0 I - c1 D
+    auto product = [&](auto vec, auto f) {
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+            const int x0 = (tile % ntx) * kTX, y0 = (tile / ntx) * kTY;
+            __syncthreads();
+            for (int q = threadIdx.x; q < (kTX + 2) * (kTY + 2); q += kPsThreads) {
+                const int cy = q / (kTX + 2), cx = q - cy * (kTX + 2);
+                const int q1 = x0 - 1 + cx, q2 = y0 - 1 + cy;
+                if (q1 < 0 || q2 < 0 || q1 > N || q2 > N) continue;
+                const bool own = cx >= 1 && cx <= kTX && cy >= 1 && cy <= kTY;
+                sv[cy][cx] = vec((size_t)q2 * n1 + q1, own);
+            }
+            __syncthreads();
+            const int m1 = x0 + tx, m2 = y0 + ty;
+            if (m1 > N || m2 > N) continue;
+            double d2x = 0.0, d2y = 0.0, mix = 0.0;
+#pragma unroll
+            for (int i = -1; i <= 1; ++i) {
+                const int c1 = clampi(m1 + i, N) - m1 + tx + 1, c2 = clampi(m2 + i, N) - m2 + ty + 1;
+                d2x += a.d.b2[m1 * 3 + i + 1] * sv[ty + 1][c1];
+                d2y += a.d.b2[m2 * 3 + i + 1] * sv[c2][tx + 1];
+                const double a2 = a.d.a1[m2 * 3 + i + 1];
+                if (a2 != 0.0) {
+#pragma unroll
+                    for (int j = -1; j <= 1; ++j)
+                        mix += a2 * a.d.a1[m1 * 3 + j + 1] * sv[c2][clampi(m1 + j, N) - m1 + tx + 1];
+                }
+            }
+            const double x1 = a.d.x[m1], x2 = a.d.x[m2];
+            const double dv = 0.5 * a.d.A11 * x1 * x1 * d2x + a.d.A12 * x1 * x2 * mix + 0.5 * a.d.A22 * x2 * x2 * d2y;
+            const double c = sv[ty + 1][tx + 1];
+            f((size_t)m2 * n1 + m1, a.c0 * c - a.c1 * dv, c);
+        }
+    };
+    // the block's own nodes
+    auto own_nodes = [&](auto f) {
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+            const int m1 = (tile % ntx) * kTX + tx, m2 = (tile / ntx) * kTY + ty;
+            if (m1 <= N && m2 <= N) f((size_t)m2 * n1 + m1);
+        }
+    };
+    PsBicg q{};
+    q.rho = q.alpha = q.omega = 1.0;
+    double acc[3] = {0.0, 0.0, 0.0};
+    product([&](size_t i, bool) { return a.X[i]; },
+            [&](size_t i, double av, double) {
+                const double b = a.B[i], r = b - av;
+                a.r[i] = r;
+                a.rh[i] = r;
+                acc[0] += b * b;
+                acc[1] += r * r;
+            });
+    if (!ps_grid_sum<2>(acc, a.part + 6 * (size_t)gridDim.x, a.st, gen)) return;
+    const double bn = sqrt(acc[0]);
+    q.lim = 1e-13 * (bn > 0.0 ? bn : 1.0);
+    q.rn = sqrt(acc[1]);
+    q.rho_new = acc[1];
+    while (q.rn > q.lim && q.it < a.maxit) {
+        // the old p and v are read at neighbours while the new ones are written: two of each
+        double* const pn = q.it & 1 ? a.p1 : a.p0;
+        double* const vn = q.it & 1 ? a.v1 : a.v0;
+        const double* const po = q.it & 1 ? a.p0 : a.p1;
+        const double* const vo = q.it & 1 ? a.v0 : a.v1;
+        const double beta = (q.rho_new / q.rho) * (q.alpha / q.omega), bo = -beta * q.omega;
+        const bool first = q.it == 0;
+        acc[0] = 0.0;
+        product([&](size_t i, bool own) {
+                    double p = __ldcg(a.r + i);
+                    if (!first) p = p + beta * __ldcg(po + i) + bo * __ldcg(vo + i);
+                    if (own) pn[i] = p;
+                    return p * a.dinv[i];
+                },
+                [&](size_t i, double av, double) {
+                    vn[i] = av;
+                    acc[0] += a.rh[i] * av;
+                });
+        if (!ps_grid_sum<1>(acc, a.part, a.st, gen)) return;
+        q.alpha = q.rho_new / acc[0];
+        acc[0] = acc[1] = acc[2] = 0.0;
+        product([&](size_t i, bool own) {
+                    const double sn = __ldcg(a.r + i) - q.alpha * __ldcg(vn + i);
+                    if (own) a.s[i] = sn;
+                    return sn * a.dinv[i];
+                },
+                [&](size_t i, double av, double) {
+                    const double sn = a.s[i];         // written by this block, before the tile's barrier
+                    a.t[i] = av;
+                    acc[0] += av * sn;
+                    acc[1] += av * av;
+                    acc[2] += sn * sn;
+                });
+        // (three regions of partial sums in turn: a block may still be reading the previous ones)
+        if (!ps_grid_sum<3>(acc, a.part + 3 * (size_t)gridDim.x, a.st, gen)) return;
+        q.it += 1;
+        const double sn = sqrt(acc[2]);
+        if (sn <= q.lim) {
+            q.rn = sn;
+            q.done = 1;
+            own_nodes([&](size_t i) { a.X[i] = a.X[i] + q.alpha * (pn[i] * a.dinv[i]); });
+            break;
+        }
+        q.omega = acc[0] / acc[1];
+        acc[0] = acc[1] = 0.0;
+        own_nodes([&](size_t i) {
+            const double di = a.dinv[i], s = a.s[i];
+            a.X[i] = a.X[i] + q.alpha * (pn[i] * di) + q.omega * (s * di);
+            const double r = s - q.omega * a.t[i];
+            a.r[i] = r;
+            acc[0] += r * r;
+            acc[1] += a.rh[i] * r;
+        });
+        if (!ps_grid_sum<2>(acc, a.part + 6 * (size_t)gridDim.x, a.st, gen)) return;
+        q.rho = q.rho_new;
+        q.rn = sqrt(acc[0]);
+        q.rho_new = acc[1];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.st->rn = q.rn;
+        a.st->lim = q.lim;
+        a.st->it = q.it;
+        a.st->done = q.done;
+    }
+}
+
+// blocks of the solve: one per tile, as many as are resident together (0 on error)
+int ps_bicg_blocks(int n1) {
+    int dev = 0, sms = 0, per = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ps_bicg, kPsThreads, 0) != cudaSuccess)
+        return 0;
+    const int tiles = ((n1 + kTX - 1) / kTX) * ((n1 + kTY - 1) / kTY);
+    return std::min(std::min(tiles, per * sms), kPsRedBlocks);
+}
+
+cudaError_t launch_ps_bicg(const PsBicgArgs& a, int blocks, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(a.st, 0, sizeof(PsBicg), s);
+    if (e != cudaSuccess) return e;
+    PsBicgArgs b = a;
+    void* args[] = {&b};
+    return cudaLaunchCooperativeKernel((const void*)k_ps_bicg, dim3(blocks), dim3(kPsThreads), args, 0, s);
 }
 
 cudaError_t launch_ps_maxrel(size_t n, const double* a, const double* b, double* part, double* res, cudaStream_t s) {
     k_ps_maxrel<<<kPsRedBlocks, 256, 0, s>>>(n, a, b, part);
-    k_ps_finish<<<1, 256, 0, s>>>(part, kPsRedBlocks, 1, 1, res);
+    k_ps_finish<<<1, 256, 0, s>>>(part, kPsRedBlocks, res);
     return cudaGetLastError();
 }
 
