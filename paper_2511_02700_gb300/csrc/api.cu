@@ -2223,7 +2223,7 @@ void price_layout(pide2d_price* H) {
     H->off_tin_w = take((size_t)H->nin * 4 * 8);
     H->off_tout_t = take((size_t)H->nx1 * 4);
     H->off_tout_u = take((size_t)H->nx1 * 4 * 8);
-    H->off_A = take((size_t)P * P * sizeof(R));
+    H->off_A = take((size_t)H->nx1 * H->nin * 8);       // T_in along axis 1
     H->off_S = take((size_t)ng * P * cgroup_bytes<R>());
     H->off_By = take((size_t)H->nout * H->nout * 8);
     H->off_loop = o;                // the time-loop fields follow (ps_loop_bytes)
@@ -2324,11 +2324,13 @@ template <typename R>
 static pide2d_status price_apply(pide2d_price* H, const double* V, double* out) {
     cudaStream_t s = H->stream;
     const int P = H->P;
-    R* A = H->at<R>(H->off_A);
+    double* A = H->at<double>(H->off_A);
     void* S = H->at<void>(H->off_S);
     const void* tw = H->at<void>(H->off_twr);
-    PIDE_PCUDA(launch_ps_tin<R>(P, H->nin, H->nx1, H->at<int>(H->off_tin_s), H->at<double>(H->off_tin_w), V, A, s));
-    PIDE_PCUDA(launch_ps_rows_fwd<R>(P, A, H->nin, S, tw, s));
+    const int* ts = H->at<int>(H->off_tin_s);
+    const double* tiw = H->at<double>(H->off_tin_w);
+    PIDE_PCUDA(launch_ps_tin(H->nin, H->nx1, ts, tiw, V, A, s));
+    PIDE_PCUDA(launch_ps_rows_fwd<R>(P, A, H->nin, ts, tiw, S, tw, s));
     PIDE_PCUDA(launch_ps_col<R>(P, S, H->at<void>(H->off_wh), H->nin, H->nout, tw, s));
     PIDE_PCUDA(launch_ps_rows_inv<R>(P, S, H->nout, H->at<double>(H->off_By), H->nout, tw, s));
     PIDE_PCUDA(launch_ps_tout(H->nx1, H->nout, H->at<int>(H->off_tout_t), H->at<double>(H->off_tout_u),

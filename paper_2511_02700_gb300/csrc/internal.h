@@ -177,10 +177,9 @@ int fft_units_per_block(int P, int prec_bytes);
 template <typename R> cudaError_t launch_prep_jobs(const PrepArgs<R>& a0, const PrepArgs<R>* arr, int K,
                                                   bool explicit_part, cudaStream_t s);
 // price-space jump operator (eqs. 3.12-3.17 on the paper's price grid); P x P transforms
-template <typename R> cudaError_t launch_ps_tin(int P, int nin, int nx1, const int* s, const double* w,
-                                               const double* V, R* A, cudaStream_t st);
-template <typename R> cudaError_t launch_ps_rows_fwd(int P, const R* A, int nin, void* S, const void* tw,
-                                                    cudaStream_t st);
+cudaError_t launch_ps_tin(int nin, int nx1, const int* s, const double* w, const double* V, double* A, cudaStream_t st);
+template <typename R> cudaError_t launch_ps_rows_fwd(int P, const double* A, int nin, const int* s, const double* w,
+                                                    void* S, const void* tw, cudaStream_t st);
 template <typename R> cudaError_t launch_ps_col(int P, void* S, const void* Wh, int nin, int nout, const void* tw,
                                                cudaStream_t st);
 template <typename R> cudaError_t launch_ps_rows_inv(int P, const void* S, int nout, double* By, int ldB,

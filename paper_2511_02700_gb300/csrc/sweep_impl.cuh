@@ -1671,33 +1671,14 @@ __global__ void __launch_bounds__(256) k_prep_jobs(const PrepArgs<float>* __rest
 // y_in lattice, the zero-padded correlation with Omega by row R2C, column
 // (forward, * conj(w^)/P^2, inverse) and row C2R passes, T_out back
 // ---------------------------------------------------------------------------
-// A[j2][j1] = sum_{b,c} w[j2][b] w[j1][c] V[s[j2]+b][s[j1]+c] on j < nin (s = -1: beyond x_max, 0)
-template <typename R>
-__global__ void k_ps_tin(int P, int nin, int nx1, const int* __restrict__ s, const double* __restrict__ w,
-                         const double* __restrict__ V, R* __restrict__ A) {
-    const int j1 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j2 = blockIdx.y * blockDim.y + threadIdx.y;
-    if (j1 >= P || j2 >= P) return;
-    double acc = 0.0;
-    if (j1 < nin && j2 < nin) {
-        const int a1 = s[j1], a2 = s[j2];
-        if (a1 >= 0 && a2 >= 0) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const double* row = V + (size_t)(a2 + b) * nx1 + a1;
-                double r = 0.0;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) r += w[j1 * 4 + c] * row[c];
-                acc += w[j2 * 4 + b] * r;
-            }
-        }
-    }
-    A[(size_t)j2 * P + j1] = (R)acc;
-}
-
-// rows 2p, 2p+1 of A (rows and columns >= nin are zero): packed R2C into S [group][row][c]
+// rows 2p, 2p+1 of T_in V on j < nin (zero beyond): packed R2C into S [group][row][c].
+// T_in along axis 1 comes in A[m2][j1] (k_ps_tin), the four taps along axis 2 are taken in
+// the first stage, where their FP64 instructions overlap the transform's integer ones; a
+// tensor product per lattice point in a kernel of its own, with a zeroed P x P array between,
+// took 215 of 2400 us for one application at N_x = 320 (nin = 3083).
 template <typename R, int P>
-PIDE_FFT_KERNEL(R, P) k_ps_rows_fwd(const R* __restrict__ A, int nin, void* Sv, int rows, int ng, const void* twv) {
+PIDE_FFT_KERNEL(R, P) k_ps_rows_fwd(const double* __restrict__ A, int nin, const int* __restrict__ ts,
+                                    const double* __restrict__ tw2, void* Sv, int rows, int ng, const void* twv) {
     using C = cpx<R>;
     using CF = Cfg<R, P>;
     constexpr int NT = CF::NT;
@@ -1708,13 +1689,29 @@ PIDE_FFT_KERNEL(R, P) k_ps_rows_fwd(const R* __restrict__ A, int nin, void* Sv, 
     const int rho = 2 * p;
     const bool valid = rho < nin;
     const C* tw = (const C*)twv;
+    // taps of the two rows (none beyond x_max)
+    const int sa = valid ? ts[rho] : -1, sb = valid && rho + 1 < nin ? ts[rho + 1] : -1;
+    const double* Ra = A + (size_t)(sa >= 0 ? sa : 0) * nin;
+    const double* Rb = A + (size_t)(sb >= 0 ? sb : 0) * nin;
+    double wa[4], wb[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        wa[b] = sa >= 0 ? tw2[rho * 4 + b] : 0.0;
+        wb[b] = sb >= 0 ? tw2[(rho + 1) * 4 + b] : 0.0;
+    }
     auto load = [&](int i) -> C {
-        R xa = 0, xb = 0;
-        if (valid && i < nin) {
-            xa = A[(size_t)rho * P + i];
-            if (rho + 1 < nin) xb = A[(size_t)(rho + 1) * P + i];
+        double xa = 0.0, xb = 0.0;
+        if (i < nin) {
+            if (sa >= 0) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) xa += wa[b] * Ra[(size_t)b * nin + i];
+            }
+            if (sb >= 0) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) xb += wb[b] * Rb[(size_t)b * nin + i];
+            }
         }
-        return mk<R>(xa, xb);
+        return mk<R>((R)xa, (R)xb);
     };
     block_fft<R, -1, P>(buf, t, tw, load, SmemStore<R>{buf});
     constexpr int Gc = cgroup<R>();
@@ -2196,21 +2193,15 @@ cudaError_t launch_prep(const PrepArgs<R>& a, cudaStream_t s) {
     }
 }
 template <typename R>
-cudaError_t launch_ps_tin(int P, int nin, int nx1, const int* s, const double* w, const double* V, R* A,
-                          cudaStream_t st) {
-    const dim3 blk(32, 8), grd((P + 31) / 32, (P + 7) / 8);
-    k_ps_tin<R><<<grd, blk, 0, st>>>(P, nin, nx1, s, w, V, A);
-    return cudaGetLastError();
-}
-template <typename R>
-cudaError_t launch_ps_rows_fwd(int P, const R* A, int nin, void* S, const void* tw, cudaStream_t st) {
+cudaError_t launch_ps_rows_fwd(int P, const double* A, int nin, const int* ts, const double* w, void* S, const void* tw,
+                               cudaStream_t st) {
     const int rows = P, ng = spectrum_groups<R>(P);
 #define CASE(PP)                                                                                     \
     if constexpr (LoopSize<R, PP>::ok) {                                                             \
         using CF = Cfg<R, PP>;                                                                       \
         set_smem(k_ps_rows_fwd<R, PP>, CF::SMEM);                                                    \
         const int units = (nin + 1) / 2;                                                             \
-        k_ps_rows_fwd<R, PP><<<(units + CF::UNITS - 1) / CF::UNITS, CF::THREADS, CF::SMEM, st>>>(A, nin, S, rows, ng, tw); \
+        k_ps_rows_fwd<R, PP><<<(units + CF::UNITS - 1) / CF::UNITS, CF::THREADS, CF::SMEM, st>>>(A, nin, ts, w, S, rows, ng, tw); \
         return cudaGetLastError();                                                                   \
     } else return cudaErrorInvalidValue;
     PIDE_SWITCH_P(P, CASE)
