@@ -334,18 +334,17 @@ static pide2d_status record_theta_step(pide2d* H, int res, double theta, double 
 
 // ---------------------------------------------------------------------------
 // the fixed-point loop of one theta step as a CUDA graph:
-//   reset(FpCtl.k, FpCtl.conv) -> while(cond) { col_solve, dst_row, check, col, inv } -> tally
-// k_fp_check clears the condition at convergence, at kmax or on a non-finite
+//   while(cond) { col_solve, dst_row (with the stopping rule), col, inv }
+// The row DST pass clears the condition at convergence, at kmax or on a non-finite
 // residual, so every launch of the graph ends.
 // ---------------------------------------------------------------------------
 namespace {
 constexpr size_t kMaxLoopGraphs = 24;
 
 template <typename R>
-cudaError_t record_loop_graph(pide2d* H, cudaGraph_t g, const ColSolveArgs<R>& da, const DstRowArgs<R>& ra,
+cudaError_t record_loop_graph(pide2d* H, cudaGraph_t g, const ColSolveArgs<R>& da, const DstRowArgs<R>& ra0,
                               const ColArgs<R>& ca, const InvArgs<R>& ia, const char** where) {
     cudaStream_t cs = H->cap;
-    FpCtl* ctl = H->at<FpCtl>(R_CTL);
     cudaError_t e = cudaSuccess;
 #define PIDE_GTRY(call)              \
     do {                             \
@@ -357,32 +356,23 @@ cudaError_t record_loop_graph(pide2d* H, cudaGraph_t g, const ColSolveArgs<R>& d
     } while (0)
     cudaGraphConditionalHandle hnd;
     PIDE_GTRY(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault));
-    cudaMemsetParams mp{};
-    mp.dst = ctl;                  // FpCtl.k and FpCtl.conv
-    mp.value = 0;
-    mp.elementSize = 4;
-    mp.width = 2;
-    mp.height = 1;
-    cudaGraphNode_t reset = nullptr, loop = nullptr;
-    PIDE_GTRY(cudaGraphAddMemsetNode(&reset, g, nullptr, 0, &mp));
+    cudaGraphNode_t loop = nullptr;
     cudaGraphNodeParams cp{};
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.handle = hnd;
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
-    PIDE_GTRY(cudaGraphAddNode(&loop, g, &reset, nullptr, 1, &cp));
+    PIDE_GTRY(cudaGraphAddNode(&loop, g, nullptr, nullptr, 0, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
+    DstRowArgs<R> ra = ra0;
+    ra.cond = (unsigned long long)hnd;
 
     // body: one iteration of the increment form of eq. 3.24
     PIDE_GTRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     auto iteration = [&]() -> cudaError_t {
         cudaError_t x;
         if ((x = launch_col_solve<R>(da, cs)) != cudaSuccess) return x;
-        if ((x = cudaMemsetAsync(H->at<void>(R_RESID), 0, 16, cs)) != cudaSuccess) return x;
         if ((x = launch_dst_row<R>(ra, cs)) != cudaSuccess) return x;
-        if ((x = launch_fp_check<R>(H->at<void>(R_RESID), ctl, H->tol, H->kmax, (unsigned long long)hnd, cs)) !=
-            cudaSuccess)
-            return x;
         if ((x = launch_col<R>(ca, cs)) != cudaSuccess) return x;
         return launch_row_inverse<R>(ia, cs);
     };
@@ -391,13 +381,6 @@ cudaError_t record_loop_graph(pide2d* H, cudaGraph_t g, const ColSolveArgs<R>& d
     const cudaError_t e2 = cudaStreamEndCapture(cs, &got);
     if (e != cudaSuccess) { *where = "loop body launches"; return e; }
     if (e2 != cudaSuccess) { *where = "cudaStreamEndCapture(body)"; return e2; }
-
-    // after the loop: fold the step's count into the statistics
-    PIDE_GTRY(cudaStreamBeginCaptureToGraph(cs, g, &loop, nullptr, 1, cudaStreamCaptureModeRelaxed));
-    e = launch_fp_tally(ctl, cs);
-    const cudaError_t e3 = cudaStreamEndCapture(cs, &got);
-    if (e != cudaSuccess) { *where = "launch_fp_tally"; return e; }
-    if (e3 != cudaSuccess) { *where = "cudaStreamEndCapture"; return e3; }
 #undef PIDE_GTRY
     return cudaSuccess;
 }
@@ -530,7 +513,6 @@ struct SolveSpec {
     const void* Wh;
     const void* Whi;
     double theta, ht;
-    int step_end;
     bool device_loop;
 };
 
@@ -655,8 +637,6 @@ static pide2d_status fixed_point_solve(pide2d* H, const SolveSpec<R>& sp, int* i
     *conv_out = false;
     SolveArgs<R> A;
     build_solve_args<R>(H, sp, &A);
-    St<R>* Y = sp.Y;
-    St<R>* BY = sp.BY;
     // B_w Y^{0} by a full sweep and the first residual
     PIDE_LAUNCH(PIDE2D_KERNEL_ROW_FORWARD_FULL, launch_row_forward<R>(A.fa, H->stream));
     PIDE_LAUNCH(PIDE2D_KERNEL_COL_FULL, launch_col<R>(A.caf, H->stream));
@@ -668,9 +648,13 @@ static pide2d_status fixed_point_solve(pide2d* H, const SolveSpec<R>& sp, int* i
 
     if (sp.device_loop) {
         // the iteration loop runs on the device (graph while-node); the step's
-        // fields Y and B_w Y are passed through FpCtl, so the graph depends on
-        // h_t and theta only; statistics are kept in FpCtl
+        // fields Y and B_w Y are passed through FpCtl (by the step's preparation), so the
+        // graph depends on h_t and theta only; statistics are kept in FpCtl
         FpCtl* ctl = H->at<FpCtl>(R_CTL);
+        ra.ctl = ctl;
+        ra.tol = H->tol;
+        ra.kmax = H->kmax;
+        ra.resid = H->at<double>(R_RESID) + 1;     // zero between passes; [0] is the host loop's
         ia.do_resid = 1;
         ia.conv_flag = &ctl->conv;
         ia.BY = nullptr;
@@ -680,7 +664,6 @@ static pide2d_status fixed_point_solve(pide2d* H, const SolveSpec<R>& sp, int* i
         cudaGraphExec_t ex = nullptr;
         const pide2d_status gs = loop_graph<R>(H, da, ra, ca, ia, &ex);
         if (gs != PIDE2D_OK) return gs;
-        PIDE_CUDA(launch_fp_setup(ctl, Y, BY, sp.step_end, H->stream));
         PIDE_CUDA(cudaGraphLaunch(ex, H->stream));
         H->ctl_dirty = true;
         *iters_out = 0;
@@ -724,7 +707,7 @@ static pide2d_status fixed_point_solve(pide2d* H, const SolveSpec<R>& sp, int* i
 // into pa, the implicit solve into sp
 template <typename R>
 static pide2d_status build_theta_step(pide2d* H, const int* list, int cnt, double theta, double ht, double tau_prev,
-                                      double tau, int res, int step_end, PrepArgs<R>* pa_out, SolveSpec<R>* sp_out) {
+                                      double tau, int res, PrepArgs<R>* pa_out, SolveSpec<R>* sp_out) {
     const Geometry g = H->L.g;
     const int N = g.N;
     const double hg = H->h;
@@ -795,7 +778,6 @@ static pide2d_status build_theta_step(pide2d* H, const int* list, int cnt, doubl
     sp.Whi = H->at<void>(R_WHI);
     sp.theta = theta;
     sp.ht = ht;
-    sp.step_end = step_end;
     sp.device_loop = !H->host_loop && !H->prof && !H->force_host_loop;
     return PIDE2D_OK;
 }
@@ -807,8 +789,13 @@ static pide2d_status theta_step(pide2d* H, const int* list, int cnt, double thet
     PrepArgs<R> pa;
     SolveSpec<R> sp;
     {
-        const pide2d_status bs = build_theta_step<R>(H, list, cnt, theta, ht, tau_prev, tau, res, step_end, &pa, &sp);
+        const pide2d_status bs = build_theta_step<R>(H, list, cnt, theta, ht, tau_prev, tau, res, &pa, &sp);
         if (bs != PIDE2D_OK) return bs;
+    }
+    if (sp.device_loop) {
+        pa.ctl = H->at<FpCtl>(R_CTL);
+        pa.BY = sp.BY;
+        pa.step_end = step_end;
     }
     PIDE_LAUNCH(PIDE2D_KERNEL_PREP, launch_prep<R>(pa, H->stream));
     int k = 0;
@@ -1300,7 +1287,6 @@ template <typename R>
 static pide2d_status do_iteration_probe(pide2d* H, const double* r, double ht, double theta, double* delta_out,
                                         double* bdelta_out, double* stop_out) {
     const Geometry g = H->L.g;
-    const int N = g.N;
     cudaStream_t s = H->stream;
     St<R>* Y = H->at<St<R>>(R_X);
     St<R>* BY = H->at<St<R>>(R_W);
@@ -1321,7 +1307,6 @@ static pide2d_status do_iteration_probe(pide2d* H, const double* r, double ht, d
     sp.Whi = H->at<void>(R_WHI);
     sp.theta = theta;
     sp.ht = ht;
-    sp.step_end = 0;
     sp.device_loop = false;
     SolveArgs<R> A;
     build_solve_args<R>(H, sp, &A);
@@ -1533,7 +1518,7 @@ static pide2d_status group_solve(pide2d* const* hs, int K, char* scratch, int up
                 PrepArgs<R> pa;
                 SolveSpec<R> sp;
                 const pide2d_status bs =
-                    build_theta_step<R>(H, list, cnt, theta, ht, tau_prev, tau, res, step_end[t], &pa, &sp);
+                    build_theta_step<R>(H, list, cnt, theta, ht, tau_prev, tau, res, &pa, &sp);
                 if (bs != PIDE2D_OK) return fail(H, bs);
                 SolveArgs<R> A;
                 build_solve_args<R>(H, sp, &A);
@@ -2030,7 +2015,6 @@ static pide2d_status do_adjoint(pide2d* H, const pide2d_model* dirs, int ndirs, 
             sp.Whi = whif;
             sp.theta = m.theta;
             sp.ht = m.ht;
-            sp.step_end = 1;
             sp.device_loop = false;
             int k = 0;
             double r = 0.0;

@@ -39,6 +39,25 @@ struct Geometry {
     int eoff;          // index offset of node m in the exp tables (N/2 + 3)
 };
 
+// state of the device-side fixed-point loop (loop_ctl.cu); the last block of the row DST pass
+// applies the stopping rule and keeps the statistics
+struct FpCtl {
+    int k;                   // iterations of the current theta step (0 between steps)
+    int conv;                // 1 once the eq. 3.25 test passed in the current step
+    int total;               // iterations over all steps run by the device loop
+    int step_k;              // iterations of the current time step (the damped step has four theta steps)
+    int max_step;            // largest per-time-step count
+    int last_step_k;         // count of the last completed time step
+    int nonconv;             // theta steps that stopped at kmax or on a non-finite residual
+    int substeps;            // theta steps run by the device loop
+    double last_resid;       // last eq. 3.25 quantity
+    double step_resid;       // its value at the end of the last completed time step
+    void* Y;                 // fields of the current theta step (the loop graph reads them here)
+    void* BY;
+    int step_end;            // 1 if the current theta step ends a time step
+    unsigned arrived;        // blocks of the row DST pass that have added their maximum (0 between passes)
+};
+
 template <typename R> struct FwdArgs {
     Geometry g;
     int mode;
@@ -101,6 +120,11 @@ template <typename R> struct DstRowArgs {
     void* resid;             // FP64 max of |D| / max(1, |Y|) (eq. 3.25), as unsigned 64-bit bits
     void* S;                 // spectrum rows of the increment (R2C), cpx<R>
     const void* tw;
+    // device-side loop (NULL otherwise): the last block applies eq. 3.25 and ends the loop
+    FpCtl* ctl;
+    double tol;
+    int kmax;
+    unsigned long long cond; // the loop's graph condition
 };
 
 template <typename R> struct PrepArgs {
@@ -122,6 +146,10 @@ template <typename R> struct PrepArgs {
     double Kd_prev, Kd_now;  // K e^{-r tau_{n-1}}, K e^{-r tau_n}
     float Kdp_h, Kdp_l, Kdn_h, Kdn_l;        // the same as double-float pairs
     int payoff;
+    // device-side loop (NULL otherwise): the step's fields for the loop's kernels
+    FpCtl* ctl;
+    St<R>* BY;
+    int step_end;
 };
 
 // Multi-job launches: grid dimension y (z for the 2D node kernels) indexes
@@ -237,22 +265,6 @@ template <typename R> cudaError_t launch_greeks(const Geometry& g, const St<R>* 
 template <typename R> cudaError_t launch_state_to_double(const Geometry& g, const St<R>* src, double* dst,
                                                         int ld_dst, int lo, cudaStream_t s);
 
-// device-side fixed-point loop control (loop_ctl.cu)
-struct FpCtl {
-    int k;                   // iterations of the current theta step (reset per step)
-    int conv;                // 1 once the eq. 3.25 test passed in the current step
-    int total;               // iterations over all steps run by the device loop
-    int step_k;              // iterations of the current time step (the damped step has four theta steps)
-    int max_step;            // largest per-time-step count
-    int last_step_k;         // count of the last completed time step
-    int nonconv;             // theta steps that stopped at kmax or on a non-finite residual
-    int substeps;            // theta steps run by the device loop
-    double last_resid;       // last eq. 3.25 quantity
-    double step_resid;       // its value at the end of the last completed time step
-    void* Y;                 // fields of the current theta step (the loop graph reads them here)
-    void* BY;
-    int step_end;            // 1 if the current theta step ends a time step
-};
 // discrete adjoint (adjoint.cu)
 struct SlWeights {
     double w1[4], w2[4];     // departure weights per axis (eq. 3.22)
@@ -291,9 +303,6 @@ template <typename R> cudaError_t launch_field_to_r(const Geometry& g, const dou
 template <typename R> cudaError_t launch_sl_shift_dots(const Geometry& g, const SlShiftArgs<R>& a, double* part,
                                                       double* acc, double scale, cudaStream_t s);
 
-template <typename R> cudaError_t launch_fp_check(const void* resid, FpCtl* ctl, double tol, int kmax,
-                                                 unsigned long long cond_handle, cudaStream_t s);
-cudaError_t launch_fp_tally(FpCtl* ctl, cudaStream_t s);
 
 // multi-job loop control (loop_ctl.cu)
 struct JobCheck {
@@ -329,7 +338,6 @@ cudaError_t launch_step_select(const void* blobs, size_t bytes, JobsState st, vo
 // graph condition `cond` after `steps` theta steps; step_end[t] = 1 if theta step t ends a time step
 cudaError_t launch_step_tally(int K, JobsState st, const int* step_end, int steps, unsigned long long cond,
                               cudaStream_t s);
-cudaError_t launch_fp_setup(FpCtl* ctl, void* Y, void* BY, int step_end, cudaStream_t s);
 
 // precompute (precompute.cu)
 struct LevyParams {
