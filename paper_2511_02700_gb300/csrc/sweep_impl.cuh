@@ -96,11 +96,39 @@ __device__ __forceinline__ R diff_state(const S* Y, size_t idx, int ld, R d11, R
 // The mixed difference of D at (row, x) is f(x + 1) - f(x - 1) with
 // f(x) = D[row + 1][x] - D[row - 1][x] (dcol below).
 
-// |d| / max(1, |y|) to select the node of a block's eq. 3.25 maximum: in FP32
-// the fast division (2 ulp; max(1, |y|) stays far below 2^126), since the
-// selected node is evaluated again in FP64; in FP64 the exact quotient
-__device__ __forceinline__ float stop_ratio(float d, float y) { return __fdividef(fabsf(d), fmaxf(1.f, fabsf(y))); }
-__device__ __forceinline__ double stop_ratio(double d, double y) { return fabs(d) / fmax(1.0, fabs(y)); }
+// A thread's node with the largest |d| / max(1, |y|) (eq. 3.25).  In FP32 the fast
+// division (2 ulp; max(1, |y|) stays far below 2^126), since the selected node is evaluated
+// again in FP64.  In FP64 ratios are compared by products, three FP64 instructions a node
+// instead of about twenty with a quotient (two FP64 lanes per SM), and one quotient is
+// formed at the end; max(1, |y|) and the test for NaN run on the integer pipe.  A NaN
+// ratio or y marks the block non-finite.
+template <typename R> struct StopSel;
+template <> struct StopSel<float> {
+    float q = -1.f, d = 0.f;
+    float2 y = make_float2(0.f, 0.f);
+    bool bad = false;
+    __device__ __forceinline__ void add(float dn, float2 yn) {
+        const float yr = st_r(yn);
+        const float r = __fdividef(fabsf(dn), fmaxf(1.f, fabsf(yr)));
+        bad |= !(r == r) || !(yr == yr);
+        if (r > q) { q = r; d = dn; y = yn; }
+    }
+    __device__ __forceinline__ float ratio() const { return q; }
+};
+template <> struct StopSel<double> {
+    double d = -1.0, m = 1.0, y = 0.0;       // |d| of the selected node (-1: none), max(1, |y|), y
+    bool bad = false;
+    static __device__ __forceinline__ bool is_nan(double x) {
+        return (unsigned)(__double2hiint(x) & 0x7fffffff) + (__double2loint(x) != 0 ? 1u : 0u) > 0x7ff00000u;
+    }
+    __device__ __forceinline__ void add(double dn, double yn) {
+        const double a = fabs(dn);
+        const double mn = (__double2hiint(yn) & 0x7fffffff) < 0x3ff00000 ? 1.0 : fabs(yn);
+        bad |= is_nan(dn) || is_nan(yn);
+        if (a * m > d * mn) { d = a; m = mn; y = yn; }
+    }
+    __device__ __forceinline__ double ratio() const { return d < 0.0 ? -1.0 : d / m; }
+};
 
 // a warp's candidate for the eq. 3.25 maximum (shared-memory reduction slot)
 struct StopCand {
@@ -1217,14 +1245,10 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
         return i <= N ? e : mk<R>(-e.x, -e.y);
     };
     St<R>* const Yv = a.Yind ? *a.Yind : a.Y;
-    // eq. 3.25: the thread's largest ratio |D| / max(1, |Y|) in the transform
-    // precision selects a node, whose D and Y are kept; the block's selected
-    // node is evaluated again in FP64 below, and that FP64 value is what the
-    // stopping rule compares with tol.  A NaN ratio or Y marks the block
-    // non-finite.
-    R qmax = R(-1), dsel = R(0);
-    St<R> ysel = st_from_r<St<R>, R>(R(0));
-    bool bad = false;
+    // eq. 3.25: the thread's largest ratio |D| / max(1, |Y|) selects a node, whose D and Y
+    // are kept; the block's selected node is evaluated again in FP64 below, and that FP64
+    // value is what the stopping rule compares with tol
+    StopSel<R> sel;
     const int ld = a.g.ldS, ldR = a.g.ldR;
     // the state rows updated after the DST arrive in L2 while it runs
     if (t == 0 && valid) l2_prefetch(Yv + (size_t)m2 * ld, (size_t)(hasb ? 2 : 1) * ld * sizeof(St<R>));
@@ -1240,10 +1264,7 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
                 const St<R> y = st_add(y0, da);
                 Yv[idx] = y;
                 a.D[(size_t)m2 * ldR + m1] = da;
-                const R yr = st_r(y);
-                const R q = stop_ratio(da, yr);
-                bad |= !(q == q) || !(yr == yr);
-                if (q > qmax) { qmax = q; dsel = da; ysel = y; }
+                sel.add(da, y);
             }
             if (hasb) {
                 db = R(0.5) * zz.x;
@@ -1251,10 +1272,7 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
                 const St<R> y = st_add(y1, db);
                 Yv[idx] = y;
                 a.D[(size_t)(m2 + 1) * ldR + m1] = db;
-                const R yr = st_r(y);
-                const R q = stop_ratio(db, yr);
-                bad |= !(q == q) || !(yr == yr);
-                if (q > qmax) { qmax = q; dsel = db; ysel = y; }
+                sel.add(db, y);
             }
         }
         buf[padi((m1 + N / 2 + 1) & (P - 1))] = mk<R>(da, db);
@@ -1293,6 +1311,9 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
     // in FP64 from its D and Y (as stored).  With FP32
     // ratios (two roundings of Y, 2 ulp of the quotient) the FP64 value found
     // is within 2^-20 relative of the exact FP64 maximum.
+    R qmax = sel.ratio(), dsel = sel.d;
+    St<R> ysel = sel.y;
+    bool bad = sel.bad;
     for (int o = 16; o > 0; o >>= 1) {
         const R oq = __shfl_xor_sync(0xffffffffu, qmax, o);
         const R od = __shfl_xor_sync(0xffffffffu, dsel, o);
