@@ -2108,7 +2108,7 @@ static pide2d_status do_adjoint(pide2d* H, const pide2d_model* dirs, int ndirs, 
 // ---------------------------------------------------------------------------
 // price-space jump operator on the paper's non-uniform price grid
 // (B_w = T_out I~ C T_in, eqs. 3.12-3.17): tables, weights and spectrum at
-// creation, five kernels per application
+// creation, three kernels per application
 // ---------------------------------------------------------------------------
 struct pide2d_price {
     pide2d_model model;
@@ -2119,7 +2119,7 @@ struct pide2d_price {
     cudaStream_t stream;
     char* ws;
     size_t off_gl, off_omega, off_pad, off_part, off_moment, off_params, off_rows, off_wh, off_twr, off_twd,
-        off_tin_s, off_tin_w, off_tout_t, off_tout_u, off_A, off_S, off_By, off_loop, total;
+        off_tin_s, off_tin_w, off_tout_t, off_tout_u, off_cin, off_cout, off_S, off_loop, total;
     std::vector<double> x;         // the price nodes
     double par[9];
     std::string err;
@@ -2182,6 +2182,8 @@ PriceSizes price_sizes(const pide2d_price_grid* g) {
     return z;
 }
 
+int even_rows(int n) { return (n + 1) & ~1; }
+
 template <typename R>
 void price_layout(pide2d_price* H) {
     const int P = H->P;
@@ -2207,9 +2209,9 @@ void price_layout(pide2d_price* H) {
     H->off_tin_w = take((size_t)H->nin * 4 * 8);
     H->off_tout_t = take((size_t)H->nx1 * 4);
     H->off_tout_u = take((size_t)H->nx1 * 4 * 8);
-    H->off_A = take((size_t)H->nx1 * H->nin * 8);       // T_in along axis 1
-    H->off_S = take((size_t)ng * P * cgroup_bytes<R>());
-    H->off_By = take((size_t)H->nout * H->nout * 8);
+    H->off_cin = sizeof(R) == 4 ? take((size_t)H->nin * 4 * 8) : H->off_tin_w;
+    H->off_cout = sizeof(R) == 4 ? take((size_t)H->nx1 * 4 * 8) : H->off_tout_u;
+    H->off_S = take((size_t)ng * even_rows(H->nx1) * cgroup_bytes<R>());    // row spectra of the price rows
     H->off_loop = o;                // the time-loop fields follow (ps_loop_bytes)
     H->total = o;
 }
@@ -2269,6 +2271,21 @@ static pide2d_status price_create(pide2d_price* H, const pide2d_price_grid* g) {
     PIDE_PCUDA(cudaMemcpyAsync(H->at<double>(H->off_tin_w), tw.data(), tw.size() * 8, cudaMemcpyHostToDevice, s));
     PIDE_PCUDA(cudaMemcpyAsync(H->at<int>(H->off_tout_t), tt.data(), tt.size() * 4, cudaMemcpyHostToDevice, s));
     PIDE_PCUDA(cudaMemcpyAsync(H->at<double>(H->off_tout_u), tu.data(), tu.size() * 8, cudaMemcpyHostToDevice, s));
+    auto pairs = [](const std::vector<double>& w) {
+        std::vector<float> p(2 * w.size());
+        for (size_t i = 0; i < w.size(); ++i) {
+            p[2 * i] = (float)w[i];
+            p[2 * i + 1] = (float)(w[i] - (double)p[2 * i]);
+        }
+        return p;
+    };
+    std::vector<float> pi, po;
+    if (sizeof(R) == 4) {
+        pi = pairs(tw);
+        po = pairs(tu);
+        PIDE_PCUDA(cudaMemcpyAsync(H->at<void>(H->off_cin), pi.data(), pi.size() * 4, cudaMemcpyHostToDevice, s));
+        PIDE_PCUDA(cudaMemcpyAsync(H->at<void>(H->off_cout), po.data(), po.size() * 4, cudaMemcpyHostToDevice, s));
+    }
     PIDE_PCUDA(launch_twiddles<R>(P, H->at<void>(H->off_twr), s));
     PIDE_PCUDA(launch_twiddles<double>(P, H->at<void>(H->off_twd), s));
     // weights on the z-lattice (N_z = nz, width hz), then conj(fft2(Omega padded))/P^2
@@ -2306,19 +2323,11 @@ static pide2d_status price_create(pide2d_price* H, const pide2d_price_grid* g) {
 
 template <typename R>
 static pide2d_status price_apply(pide2d_price* H, const double* V, double* out) {
-    cudaStream_t s = H->stream;
-    const int P = H->P;
-    double* A = H->at<double>(H->off_A);
-    void* S = H->at<void>(H->off_S);
-    const void* tw = H->at<void>(H->off_twr);
-    const int* ts = H->at<int>(H->off_tin_s);
-    const double* tiw = H->at<double>(H->off_tin_w);
-    PIDE_PCUDA(launch_ps_tin(H->nin, H->nx1, ts, tiw, V, A, s));
-    PIDE_PCUDA(launch_ps_rows_fwd<R>(P, A, H->nin, ts, tiw, S, tw, s));
-    PIDE_PCUDA(launch_ps_col<R>(P, S, H->at<void>(H->off_wh), H->nin, H->nout, tw, s));
-    PIDE_PCUDA(launch_ps_rows_inv<R>(P, S, H->nout, H->at<double>(H->off_By), H->nout, tw, s));
-    PIDE_PCUDA(launch_ps_tout(H->nx1, H->nout, H->at<int>(H->off_tout_t), H->at<double>(H->off_tout_u),
-                              H->at<double>(H->off_By), H->nout, out, s));
+    const PsInterp ip{H->nx1, even_rows(H->nx1), H->nin, H->at<int>(H->off_tin_s), H->at<double>(H->off_tin_w),
+                      H->at<int>(H->off_tout_t), H->at<double>(H->off_tout_u), H->at<void>(H->off_cin),
+                      H->at<void>(H->off_cout)};
+    PIDE_PCUDA(launch_ps_apply<R>(H->P, V, ip, H->at<void>(H->off_S), H->at<void>(H->off_wh), out,
+                                  H->at<void>(H->off_twr), H->stream));
     return PIDE2D_OK;
 }
 

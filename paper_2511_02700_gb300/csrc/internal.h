@@ -205,15 +205,17 @@ int fft_units_per_block(int P, int prec_bytes);
 template <typename R> cudaError_t launch_prep_jobs(const PrepArgs<R>& a0, const PrepArgs<R>* arr, int K,
                                                   bool explicit_part, cudaStream_t s);
 // price-space jump operator (eqs. 3.12-3.17 on the paper's price grid); P x P transforms
-cudaError_t launch_ps_tin(int nin, int nx1, const int* s, const double* w, const double* V, double* A, cudaStream_t st);
-template <typename R> cudaError_t launch_ps_rows_fwd(int P, const double* A, int nin, const int* s, const double* w,
-                                                    void* S, const void* tw, cudaStream_t st);
-template <typename R> cudaError_t launch_ps_col(int P, void* S, const void* Wh, int nin, int nout, const void* tw,
-                                               cudaStream_t st);
-template <typename R> cudaError_t launch_ps_rows_inv(int P, const void* S, int nout, double* By, int ldB,
-                                                    const void* tw, cudaStream_t st);
-cudaError_t launch_ps_tout(int nx1, int nout, const int* t, const double* u, const double* By, int ldB, double* out,
-                           cudaStream_t st);
+struct PsInterp {
+    int n1, rows;            // price nodes per axis; the same rounded up to even
+    int nin;                 // T_in: lattice points, first tap (-1: beyond x_max) and four weights of each
+    const int* ts;
+    const double* tw;
+    const int* to;           // T_out: first tap on the y_out lattice and four weights of each price node
+    const double* uo;
+    const void *ctw, *cuo;   // the weights as the column pass takes them: doubles, or (high, low) float pairs
+};
+template <typename R> cudaError_t launch_ps_apply(int P, const double* V, const PsInterp& ip, void* S, const void* Wh,
+                                                 double* out, const void* tw, cudaStream_t st);
 // price-space diffusion and the Krylov solve around it (price_space.cu), FP64
 struct PsDiff {
     int n1;                  // nodes per axis

@@ -1,67 +1,8 @@
-// T_out of the price-space jump operator (eq. 3.15): from the y_out lattice
-// back to the non-uniform price grid, cubic Lagrange per axis (linear
-// extrapolation below y_out is encoded in the tables as two taps).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "internal.h"
-
-namespace pide {
-
-// T_in along axis 1: A[m2][j1] = sum_c w[j1][c] V[m2][s[j1]+c], j1 < nin (s = -1: beyond x_max, 0)
-__global__ void k_ps_tin(int nin, int nx1, const int* __restrict__ s, const double* __restrict__ w,
-                         const double* __restrict__ V, double* __restrict__ A) {
-    const int j1 = blockIdx.x * blockDim.x + threadIdx.x, m2 = blockIdx.y * blockDim.y + threadIdx.y;
-    if (j1 >= nin || m2 >= nx1) return;
-    const int a1 = s[j1];
-    double r = 0.0;
-    if (a1 >= 0) {
-        const double* row = V + (size_t)m2 * nx1 + a1;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) r += w[j1 * 4 + c] * row[c];
-    }
-    A[(size_t)m2 * nin + j1] = r;
-}
-
-cudaError_t launch_ps_tin(int nin, int nx1, const int* s, const double* w, const double* V, double* A, cudaStream_t st) {
-    const dim3 blk(32, 8), grd((nin + 31) / 32, (nx1 + 7) / 8);
-    k_ps_tin<<<grd, blk, 0, st>>>(nin, nx1, s, w, V, A);
-    return cudaGetLastError();
-}
-
-__global__ void k_ps_tout(int nx1, int nout, const int* __restrict__ t, const double* __restrict__ u,
-                          const double* __restrict__ By, int ldB, double* __restrict__ out) {
-    const int m1 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int m2 = blockIdx.y * blockDim.y + threadIdx.y;
-    if (m1 >= nx1 || m2 >= nx1) return;
-    const int a1 = t[m1], a2 = t[m2];
-    double acc = 0.0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        const double wb = u[m2 * 4 + b];
-        if (wb == 0.0) continue;
-        const double* row = By + (size_t)(a2 + b) * ldB + a1;
-        double r = 0.0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const double wc = u[m1 * 4 + c];
-            if (wc != 0.0) r += wc * row[c];
-        }
-        acc += wb * r;
-    }
-    out[(size_t)m2 * nx1 + m1] = acc;
-}
-
-cudaError_t launch_ps_tout(int nx1, int nout, const int* t, const double* u, const double* By, int ldB, double* out,
-                           cudaStream_t st) {
-    (void)nout;
-    const dim3 blk(32, 8), grd((nx1 + 31) / 32, (nx1 + 7) / 8);
-    k_ps_tout<<<grd, blk, 0, st>>>(nx1, nout, t, u, By, ldB, out);
-    return cudaGetLastError();
-}
-
-}  // namespace pide
 
 // ---------------------------------------------------------------------------
 // the price-space time loop (Sec. 3.3 on the paper's grid), FP64

@@ -15,9 +15,7 @@ namespace pide {
     template cudaError_t launch_corr_col<R>(const Geometry&, const void*, const void*, int, int, double*, \
                                             const void*, cudaStream_t);                             \
     template cudaError_t launch_corr_finish<R>(const Geometry&, double*, double*, const void*, cudaStream_t); \
-    template cudaError_t launch_ps_rows_fwd<R>(int, const double*, int, const int*, const double*, void*, const void*, cudaStream_t); \
-    template cudaError_t launch_ps_col<R>(int, void*, const void*, int, int, const void*, cudaStream_t); \
-    template cudaError_t launch_ps_rows_inv<R>(int, const void*, int, double*, int, const void*, cudaStream_t); \
+    template cudaError_t launch_ps_apply<R>(int, const double*, const PsInterp&, void*, const void*, double*, const void*, cudaStream_t); \
     template cudaError_t launch_row_forward_jobs<R>(const FwdArgs<R>&, const FwdArgs<R>*, int, JobsCtl, int, cudaStream_t); \
     template cudaError_t launch_col_jobs<R>(const ColArgs<R>&, const ColArgs<R>*, int, JobsCtl, int, cudaStream_t); \
     template cudaError_t launch_row_inverse_jobs<R>(const InvArgs<R>&, const InvArgs<R>*, int, JobsCtl, int, cudaStream_t); \

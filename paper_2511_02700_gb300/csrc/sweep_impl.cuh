@@ -1738,77 +1738,74 @@ __global__ void __launch_bounds__(256) k_prep_jobs(const PrepArgs<float>* __rest
 
 // ---------------------------------------------------------------------------
 // price-space jump operator B_w = T_out I~ C T_in (eqs. 3.12-3.17 on the
-// paper's non-uniform price grid): T_in into a P x P real array on the
-// y_in lattice, the zero-padded correlation with Omega by row R2C, column
-// (forward, * conj(w^)/P^2, inverse) and row C2R passes, T_out back
+// paper's non-uniform price grid): a zero-padded P x P correlation with Omega
+// between two tensor-product interpolations.  A transform along axis 1 commutes
+// with an interpolation along axis 2, so T_in and T_out act along axis 2 inside the
+// column pass and the row passes run over the n1 price rows only, not over the nin
+// and nout lattice rows (3084 and 1805 at N_x = 320).  No lattice-sized field exists:
+// S holds n1 rows of spectra.  Against lattice rows and kernels of their own for the ends:
+// FP64 N_x = 320 866 -> 611 us, N_x = 150 (NIG) 811 -> 552 us; FP32 N_x = 320 253 -> 141 us,
+// with an eighth of the error (the lattice field was rounded before T_out's extrapolation
+// near x = 0 amplified it).  The column pass is what is left (494 of 588 us at N_x = 320,
+// 52 and 41 for the rows).
 // ---------------------------------------------------------------------------
-// rows 2p, 2p+1 of T_in V on j < nin (zero beyond): packed R2C into S [group][row][c].
-// T_in along axis 1 comes in A[m2][j1] (k_ps_tin), the four taps along axis 2 are taken in
-// the first stage, where their FP64 instructions overlap the transform's integer ones; a
-// tensor product per lattice point in a kernel of its own, with a zeroed P x P array between,
-// took 215 of 2400 us for one application at N_x = 320 (nin = 3083).
+// price rows 2p, 2p + 1: T_in along axis 1 (four taps of the row, 0 beyond x_max) in the
+// first stage, packed R2C into S [group][row][c]
 template <typename R, int P>
-PIDE_FFT_KERNEL(R, P) k_ps_rows_fwd(const double* __restrict__ A, int nin, const int* __restrict__ ts,
-                                    const double* __restrict__ tw2, void* Sv, int rows, int ng, const void* twv) {
+PIDE_FFT_KERNEL(R, P) k_ps_rows_fwd(const double* __restrict__ V, PsInterp ip, void* S, int ng, const void* twv) {
     using C = cpx<R>;
     using CF = Cfg<R, P>;
     constexpr int NT = CF::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int unit = threadIdx.x / NT, t = threadIdx.x - unit * NT;
     C* buf = reinterpret_cast<C*>(smem_raw) + (size_t)unit * CF::ULEN;
-    const int p = blockIdx.x * CF::UNITS + unit;
-    const int rho = 2 * p;
-    const bool valid = rho < nin;
+    const int rho = 2 * (blockIdx.x * CF::UNITS + unit);
+    const bool valid = rho < ip.n1, hasb = rho + 1 < ip.n1;
     const C* tw = (const C*)twv;
-    // taps of the two rows (none beyond x_max)
-    const int sa = valid ? ts[rho] : -1, sb = valid && rho + 1 < nin ? ts[rho + 1] : -1;
-    const double* Ra = A + (size_t)(sa >= 0 ? sa : 0) * nin;
-    const double* Rb = A + (size_t)(sb >= 0 ? sb : 0) * nin;
-    double wa[4], wb[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        wa[b] = sa >= 0 ? tw2[rho * 4 + b] : 0.0;
-        wb[b] = sb >= 0 ? tw2[(rho + 1) * 4 + b] : 0.0;
-    }
+    const double* Va = V + (size_t)(valid ? rho : 0) * ip.n1;
     auto load = [&](int i) -> C {
         double xa = 0.0, xb = 0.0;
-        if (i < nin) {
-            if (sa >= 0) {
+        const int s = valid && i < ip.nin ? ip.ts[i] : -1;
+        if (s >= 0) {
 #pragma unroll
-                for (int b = 0; b < 4; ++b) xa += wa[b] * Ra[(size_t)b * nin + i];
-            }
-            if (sb >= 0) {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) xb += wb[b] * Rb[(size_t)b * nin + i];
+            for (int c = 0; c < 4; ++c) {
+                const double w = ip.tw[i * 4 + c];
+                xa += w * Va[s + c];
+                if (hasb) xb += w * Va[ip.n1 + s + c];
             }
         }
         return mk<R>((R)xa, (R)xb);
     };
     block_fft<R, -1, P>(buf, t, tw, load, SmemStore<R>{buf});
-    constexpr int Gc = cgroup<R>();
-    C* S = (C*)Sv;
-    for (int g = t; g < ng; g += NT) {
-#pragma unroll
-        for (int c = 0; c < Gc; ++c) {
-            const int k = g * Gc + c;
-            C xa = mk<R>(0, 0), xb = mk<R>(0, 0);
-            if (k <= P / 2) {
-                const C zk = buf[padi(k)];
-                const C zm = buf[padi((P - k) & (P - 1))];
-                xa = mk<R>(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
-                xb = mk<R>(R(0.5) * (zk.y + zm.y), R(-0.5) * (zk.x - zm.x));
-            }
-            if (valid) {
-                S[((size_t)g * rows + rho) * Gc + c] = xa;
-                S[((size_t)g * rows + rho + 1) * Gc + c] = xb;
-            }
-        }
-    }
+    store_spectrum_rows<R, P>(buf, (C*)S, ip.rows, ng, rho, t, valid);
 }
 
-// column k1: rows < nin in, forward FFT, * Wh, inverse FFT, rows < nout out (in place)
+// column k1, in place: T_in along axis 2 in the first stage, forward FFT, * Wh, inverse FFT,
+// T_out along axis 2 (the row past an odd n1 becomes 0).  With FP64 spectra the taps are 8
+// FP64 instructions a lattice point, overlapping the transform's integer ones; with FP32 ones
+// they are summed in double-float, since FP64 products and conversions took longer than the
+// transform (N_x = 320: 284 us, double-float 141).
+template <typename R> struct TapSum;
+template <> struct TapSum<double> {
+    using W = double;
+    double s = 0.0;
+    __device__ __forceinline__ void add(double w, double z) { s += w * z; }
+    __device__ __forceinline__ double value() const { return s; }
+    static __device__ __forceinline__ bool none(double w) { return w == 0.0; }
+};
+template <> struct TapSum<float> {
+    using W = float2;                        // w.x + w.y
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float2 w, float z) {
+        const float p = w.x * z, t = s + p, b = t - s;
+        e += (s - (t - b)) + (p - b) + fmaf(w.y, z, fmaf(w.x, z, -p));
+        s = t;
+    }
+    __device__ __forceinline__ float value() const { return s + e; }
+    static __device__ __forceinline__ bool none(float2 w) { return w.x == 0.f; }
+};
 template <typename R, int P>
-PIDE_FFT_KERNEL(R, P) k_ps_col(void* Sv, const void* Whv, int rows, int nin, int nout, const void* twv) {
+PIDE_FFT_KERNEL(R, P) k_ps_col(void* Sv, const void* Whv, PsInterp ip, const void* twv) {
     using C = cpx<R>;
     using CF = Cfg<R, P>;
     constexpr int NT = CF::NT;
@@ -1819,34 +1816,60 @@ PIDE_FFT_KERNEL(R, P) k_ps_col(void* Sv, const void* Whv, int rows, int nin, int
     const bool valid = k1 <= P / 2;
     constexpr int Gc = cgroup<R>();
     const int g = k1 / Gc, c = k1 - g * Gc;
-    C* col = (C*)Sv + (size_t)g * rows * Gc + c;
+    C* col = (C*)Sv + (size_t)g * ip.rows * Gc + c;
     const C* wh = (const C*)Whv + (size_t)k1 * P;      // column-major weight spectrum
     const C* tw = (const C*)twv;
-    auto load = [&](int rho) -> C { return (valid && rho < nin) ? col[(size_t)rho * Gc] : mk<R>(0, 0); };
+    if (t == 0 && valid) l2_prefetch(wh, (size_t)P * sizeof(C));
+    using W = typename TapSum<R>::W;
+    const W *cw = (const W*)ip.ctw, *cu = (const W*)ip.cuo;
+    auto load = [&](int i) -> C {
+        TapSum<R> x, y;
+        const int s = valid && i < ip.nin ? ip.ts[i] : -1;
+        if (s >= 0) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const W w = cw[i * 4 + b];
+                const C z = col[(size_t)(s + b) * Gc];
+                x.add(w, z.x);
+                y.add(w, z.y);
+            }
+        }
+        return mk<R>(x.value(), y.value());
+    };
     auto store_mul = [&](int k2, C v) {
         const C w = valid ? __ldg(&wh[k2]) : mk<R>(0, 0);
         buf[padi(k2)] = cmul(v, w);
     };
     block_fft<R, -1, P>(buf, t, tw, load, store_mul);
-    auto store_out = [&](int m, C v) {
-        if (valid && m < nout) col[(size_t)m * Gc] = v;
-    };
-    block_fft<R, +1, P>(buf, t, tw, SmemLoad<R>{buf}, store_out);
+    block_fft<R, +1, P>(buf, t, tw, SmemLoad<R>{buf}, SmemStore<R>{buf});
+    for (int m = t; m < ip.rows && valid; m += NT) {
+        TapSum<R> x, y;
+        if (m < ip.n1) {
+            const int a = ip.to[m];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const W u = cu[m * 4 + b];
+                if (TapSum<R>::none(u)) continue;      // a linear end has two taps
+                const C z = buf[padi(a + b)];
+                x.add(u, z.x);
+                y.add(u, z.y);
+            }
+        }
+        col[(size_t)m * Gc] = mk<R>(x.value(), y.value());
+    }
 }
 
-// output rows 2p, 2p+1 (< nout): packed C2R of the Hermitian spectrum, By[row][m1] for m1 < nout
+// price rows 2p, 2p + 1: packed C2R of the Hermitian spectrum, T_out along axis 1
 template <typename R, int P>
-PIDE_FFT_KERNEL(R, P) k_ps_rows_inv(const void* Sv, int rows, int nout, double* __restrict__ By, int ldB,
-                                    const void* twv) {
+PIDE_FFT_KERNEL(R, P) k_ps_rows_inv(const void* Sv, PsInterp ip, double* __restrict__ out, const void* twv) {
     using C = cpx<R>;
     using CF = Cfg<R, P>;
     constexpr int NT = CF::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int unit = threadIdx.x / NT, t = threadIdx.x - unit * NT;
     C* buf = reinterpret_cast<C*>(smem_raw) + (size_t)unit * CF::ULEN;
-    const int p = blockIdx.x * CF::UNITS + unit;
-    const int r = 2 * p;
-    const bool valid = r < nout;
+    const int r = 2 * (blockIdx.x * CF::UNITS + unit);
+    const bool valid = r < ip.n1;
     constexpr int Gc = cgroup<R>();
     const C* S = (const C*)Sv;
     const C* tw = (const C*)twv;
@@ -1856,19 +1879,28 @@ PIDE_FFT_KERNEL(R, P) k_ps_rows_inv(const void* Sv, int rows, int nout, double* 
         C xa = mk<R>(0, 0), xb = mk<R>(0, 0);
         if (valid) {
             const int g = k / Gc, c = k - g * Gc;
-            xa = S[((size_t)g * rows + r) * Gc + c];
-            xb = S[((size_t)g * rows + r + 1) * Gc + c];
+            xa = S[((size_t)g * ip.rows + r) * Gc + c];
+            xb = S[((size_t)g * ip.rows + r + 1) * Gc + c];
         }
         if (k == 0 || k == P / 2) { xa.y = 0; xb.y = 0; }
         if (hi) { xa.y = -xa.y; xb.y = -xb.y; }
         return mk<R>(xa.x - xb.y, xa.y + xb.x);
     };
-    auto store = [&](int m1, C z) {
-        if (!valid || m1 >= nout) return;
-        By[(size_t)r * ldB + m1] = (double)z.x;
-        if (r + 1 < nout) By[(size_t)(r + 1) * ldB + m1] = (double)z.y;
-    };
-    block_fft<R, +1, P>(buf, t, tw, load, store);
+    block_fft<R, +1, P>(buf, t, tw, load, SmemStore<R>{buf});
+    for (int m = t; m < ip.n1 && valid; m += NT) {
+        const int a = ip.to[m];
+        double x = 0.0, y = 0.0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double u = ip.uo[m * 4 + c];
+            if (u == 0.0) continue;
+            const C z = buf[padi(a + c)];
+            x += u * (double)z.x;
+            y += u * (double)z.y;
+        }
+        out[(size_t)r * ip.n1 + m] = x;
+        if (r + 1 < ip.n1) out[(size_t)(r + 1) * ip.n1 + m] = y;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2264,40 +2296,19 @@ cudaError_t launch_prep(const PrepArgs<R>& a, cudaStream_t s) {
     }
 }
 template <typename R>
-cudaError_t launch_ps_rows_fwd(int P, const double* A, int nin, const int* ts, const double* w, void* S, const void* tw,
-                               cudaStream_t st) {
-    const int rows = P, ng = spectrum_groups<R>(P);
+cudaError_t launch_ps_apply(int P, const double* V, const PsInterp& ip, void* S, const void* Wh, double* out,
+                            const void* tw, cudaStream_t st) {
 #define CASE(PP)                                                                                     \
     if constexpr (LoopSize<R, PP>::ok) {                                                             \
         using CF = Cfg<R, PP>;                                                                       \
+        const int rows = (ip.rows / 2 + CF::UNITS - 1) / CF::UNITS;                                  \
+        const int cols = (PP / 2 + 1 + CF::UNITS - 1) / CF::UNITS;                                   \
         set_smem(k_ps_rows_fwd<R, PP>, CF::SMEM);                                                    \
-        const int units = (nin + 1) / 2;                                                             \
-        k_ps_rows_fwd<R, PP><<<(units + CF::UNITS - 1) / CF::UNITS, CF::THREADS, CF::SMEM, st>>>(A, nin, ts, w, S, rows, ng, tw); \
-        return cudaGetLastError();                                                                   \
-    } else return cudaErrorInvalidValue;
-    PIDE_SWITCH_P(P, CASE)
-#undef CASE
-}
-template <typename R>
-cudaError_t launch_ps_col(int P, void* S, const void* Wh, int nin, int nout, const void* tw, cudaStream_t st) {
-#define CASE(PP)                                                                                     \
-    if constexpr (LoopSize<R, PP>::ok) {                                                             \
-        using CF = Cfg<R, PP>;                                                                       \
         set_smem(k_ps_col<R, PP>, CF::SMEM);                                                         \
-        k_ps_col<R, PP><<<(PP / 2 + 1 + CF::UNITS - 1) / CF::UNITS, CF::THREADS, CF::SMEM, st>>>(S, Wh, PP, nin, nout, tw); \
-        return cudaGetLastError();                                                                   \
-    } else return cudaErrorInvalidValue;
-    PIDE_SWITCH_P(P, CASE)
-#undef CASE
-}
-template <typename R>
-cudaError_t launch_ps_rows_inv(int P, const void* S, int nout, double* By, int ldB, const void* tw, cudaStream_t st) {
-#define CASE(PP)                                                                                     \
-    if constexpr (LoopSize<R, PP>::ok) {                                                             \
-        using CF = Cfg<R, PP>;                                                                       \
         set_smem(k_ps_rows_inv<R, PP>, CF::SMEM);                                                    \
-        const int units = (nout + 1) / 2;                                                            \
-        k_ps_rows_inv<R, PP><<<(units + CF::UNITS - 1) / CF::UNITS, CF::THREADS, CF::SMEM, st>>>(S, PP, nout, By, ldB, tw); \
+        k_ps_rows_fwd<R, PP><<<rows, CF::THREADS, CF::SMEM, st>>>(V, ip, S, spectrum_groups<R>(PP), tw); \
+        k_ps_col<R, PP><<<cols, CF::THREADS, CF::SMEM, st>>>(S, Wh, ip, tw);                         \
+        k_ps_rows_inv<R, PP><<<rows, CF::THREADS, CF::SMEM, st>>>(S, ip, out, tw);                   \
         return cudaGetLastError();                                                                   \
     } else return cudaErrorInvalidValue;
     PIDE_SWITCH_P(P, CASE)
