@@ -227,8 +227,14 @@ struct PsDiff {
 cudaError_t launch_ps_diff(const PsDiff& d, const double* v, double alpha, double beta, const double* w, double gamma,
                            double* out, cudaStream_t s);
 cudaError_t launch_ps_diag_inv(const PsDiff& d, double c0, double c1, double* dinv, cudaStream_t s);
-cudaError_t launch_ps_axpy(size_t n, double a, const double* x, double b, const double* y, double c, const double* z,
-                           const double* dinv, double* out, cudaStream_t s);
+struct PsHistory {
+    int count;               // values kept, newest first, with the extrapolation's coefficients
+    double c[4];
+    const double *V[4], *BV[4];
+};
+cudaError_t launch_ps_start(size_t n, const PsHistory& h, double* Y, double* BY, cudaStream_t s);
+cudaError_t launch_ps_rhs(size_t n, double htt, const double* W, const double* ZZ, const double* Y, double* BY, double* B,
+                          double* X, cudaStream_t s);
 int ps_reduction_blocks();
 // one Jacobi-preconditioned BiCGSTAB solve of (c0 I - c1 D) X = B to a relative residual of
 // 1e-13, as one cooperative launch
@@ -252,7 +258,7 @@ struct PsBicgArgs {
 };
 int ps_bicg_blocks(int n1);
 cudaError_t launch_ps_bicg(const PsBicgArgs& a, int blocks, cudaStream_t s);
-cudaError_t launch_ps_maxrel(size_t n, const double* a, const double* b, double* part, double* res, cudaStream_t s);
+cudaError_t launch_ps_update(size_t n, const double* X, double* Y, double* T, double* part, double* res, cudaStream_t s);
 cudaError_t launch_ps_sl(int n1, const int* s1, const double* w1, const int* s2, const double* w2, const double* Z,
                          double* W, cudaStream_t s);
 // omega-hat: forward column FFT of the FP64 row spectra, written as cpx<RO>

@@ -55,25 +55,43 @@ __global__ void k_ps_diag_inv(PsDiff d, double c0, double c1, double* __restrict
     dinv[(size_t)m2 * d.n1 + m1] = 1.0 / (c0 - c1 * dd);
 }
 
-// elementwise: out = a x + b y + c z (y, z may be NULL), or with dinv: out = dinv * (a x + b y)
-// out may be one of x, y, z (each element is read before it is written): no __restrict__
-__global__ void k_ps_axpy(size_t n, double a, const double* x, double b, const double* y, double c,
-                          const double* z, const double* dinv, double* out) {
+// Y^{n,0} = sum_i c_i V^{n-i} (eq. 3.26), and, BV given, its B_w Y by the same sum of B_w V^{n-i}
+__global__ void k_ps_start(size_t n, PsHistory h, double* __restrict__ Y, double* __restrict__ BY) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double r = a * x[i];
-    if (y) r += b * y[i];
-    if (z) r += c * z[i];
-    if (dinv) r *= dinv[i];
-    out[i] = r;
+    double y = h.c[0] * h.V[0][i];
+    for (int k = 1; k < h.count; ++k) y += h.c[k] * h.V[k][i];
+    Y[i] = y;
+    if (!BY) return;
+    double b = h.c[0] * h.BV[0][i];
+    for (int k = 1; k < h.count; ++k) b += h.c[k] * h.BV[k][i];
+    BY[i] = b;
 }
 
-__global__ void k_ps_maxrel(size_t n, const double* __restrict__ a, const double* __restrict__ b,
+// before an implicit solve: B_w Y += ZZ (the jump of the last increment, or NULL), its right-hand
+// side B = h_t theta B_w Y + W, and its start X = Y
+__global__ void k_ps_rhs(size_t n, double htt, const double* __restrict__ W, const double* __restrict__ ZZ,
+                         const double* __restrict__ Y, double* __restrict__ BY, double* __restrict__ B,
+                         double* __restrict__ X) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double by = BY[i];
+    if (ZZ) BY[i] = by += ZZ[i];
+    B[i] = htt * by + W[i];
+    X[i] = Y[i];
+}
+
+// after it: the increment T = X - Y, Y = X, and eq. 3.25's maximum per block
+__global__ void k_ps_update(size_t n, const double* __restrict__ X, double* __restrict__ Y, double* __restrict__ T,
                             double* __restrict__ part) {
     __shared__ double red[256];
     double m = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        m = fmax(m, fabs(a[i] - b[i]) / fmax(1.0, fabs(a[i])));
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double x = X[i], t = x - Y[i];
+        m = fmax(m, fabs(t) / fmax(1.0, fabs(x)));
+        T[i] = t;
+        Y[i] = x;
+    }
     red[threadIdx.x] = m;
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
@@ -110,9 +128,13 @@ cudaError_t launch_ps_diag_inv(const PsDiff& d, double c0, double c1, double* di
     k_ps_diag_inv<<<grd, blk, 0, s>>>(d, c0, c1, dinv);
     return cudaGetLastError();
 }
-cudaError_t launch_ps_axpy(size_t n, double a, const double* x, double b, const double* y, double c, const double* z,
-                           const double* dinv, double* out, cudaStream_t s) {
-    k_ps_axpy<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, a, x, b, y, c, z, dinv, out);
+cudaError_t launch_ps_start(size_t n, const PsHistory& h, double* Y, double* BY, cudaStream_t s) {
+    k_ps_start<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, h, Y, BY);
+    return cudaGetLastError();
+}
+cudaError_t launch_ps_rhs(size_t n, double htt, const double* W, const double* ZZ, const double* Y, double* BY, double* B,
+                          double* X, cudaStream_t s) {
+    k_ps_rhs<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, htt, W, ZZ, Y, BY, B, X);
     return cudaGetLastError();
 }
 int ps_reduction_blocks() { return kPsRedBlocks; }
@@ -335,8 +357,8 @@ cudaError_t launch_ps_bicg(const PsBicgArgs& a, int blocks, cudaStream_t s) {
     return cudaLaunchCooperativeKernel((const void*)k_ps_bicg, dim3(blocks), dim3(kPsThreads), args, 0, s);
 }
 
-cudaError_t launch_ps_maxrel(size_t n, const double* a, const double* b, double* part, double* res, cudaStream_t s) {
-    k_ps_maxrel<<<kPsRedBlocks, 256, 0, s>>>(n, a, b, part);
+cudaError_t launch_ps_update(size_t n, const double* X, double* Y, double* T, double* part, double* res, cudaStream_t s) {
+    k_ps_update<<<kPsRedBlocks, 256, 0, s>>>(n, X, Y, T, part);
     k_ps_finish<<<1, 256, 0, s>>>(part, kPsRedBlocks, res);
     return cudaGetLastError();
 }
