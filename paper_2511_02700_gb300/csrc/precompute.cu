@@ -343,9 +343,8 @@ __global__ void k_twiddles(int P, cpx<R>* tw) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= tw_entries<R>(P)) return;
     if (sizeof(R) == 8 && i >= P) {          // the Q62 halves of w^{i - P}
-        double s, c;
-        sincospi(2.0 * (double)(i - P) / P, &s, &c);
-        const FxHalf re = fx_q62(c), im = fx_q62(-s);
+        const fx2 w = fx_twiddle(i - P, P);
+        const FxHalf re = fx_split(w.x), im = fx_split(w.y);
         reinterpret_cast<int4*>(tw)[i] = make_int4(re.h, re.l, im.h, im.l);
         return;
     }
