@@ -2083,11 +2083,26 @@ __global__ void k_state_from_double(Geometry g, const double* src, int lds, St<R
     if (m1 > g.N || m2 > g.N) return;
     dst[(size_t)m2 * g.ldS + m1] = st_make<St<R>>(src[(size_t)m2 * lds + m1]);
 }
+// float to double by integer instructions (the conversion instruction outside the normal range):
+// a warp's FP64 conversion or sum occupies the SM for 16 clocks.  N = 4096: 92 -> 59 us a field
+// with the low parts zero, now bound by memory (201 MB, of which 67 MB zeros).
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m == 0u) return __hiloint2double((int)u, 0);
+    if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
+__device__ __forceinline__ double to_double(float2 a) {
+    const double h = widen(a.x);
+    return a.y == 0.f ? h : h + widen(a.y);
+}
+
 template <typename R>
 __global__ void k_state_to_double(Geometry g, const St<R>* src, double* dst, int ldd, int lo) {
     const int m1 = blockIdx.x * blockDim.x + threadIdx.x, m2 = blockIdx.y * blockDim.y + threadIdx.y;
     if (m1 < lo || m2 < lo || m1 > g.N - lo || m2 > g.N - lo) return;
-    dst[(size_t)m2 * ldd + m1] = st_dbl(src[(size_t)m2 * g.ldS + m1]);
+    dst[(size_t)m2 * ldd + m1] = to_double(src[(size_t)m2 * g.ldS + m1]);
 }
 
 // ---------------------------------------------------------------------------
