@@ -44,7 +44,12 @@ template <typename R, int P> struct Cfg {
     static constexpr int THREADS = UNITS * NT;
     // staged columns reach two elements past the padded length; the FP64 transform's slots follow
     static constexpr int ULEN = padded_len(P) + (sizeof(R) == 8 ? 12 : 4);
-    static constexpr int TPS = sizeof(R) == 4 ? 1024 : 512;         // resident threads per SM
+    // resident threads per SM: 64 registers a thread in FP32 and in the FP64 transforms of 8 values
+    // whose passes fill the chip (P = 2048, 4096: twice the warps outweigh up to 700 bytes of
+    // spills in the inverse row pass; jump sum N = 1024 328 -> 284 us, N = 2048 1264 -> 1019 us;
+    // 85 registers at P = 2048: 265 us), 128 otherwise (P = 1024: 114 us against 120 with 64; at
+    // P = 8192 16 values a thread spill, its row pass takes 674 us against 497)
+    static constexpr int TPS = sizeof(R) == 4 || P == 2048 || P == 4096 ? 1024 : 512;
     static constexpr int MINB = TPS / THREADS < 24 ? TPS / THREADS : 24;
     static constexpr size_t SMEM = (size_t)UNITS * ULEN * sizeof(cpx<R>);
     // multi-job kernels: launched with any number of units per block up to
