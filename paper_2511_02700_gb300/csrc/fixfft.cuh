@@ -13,9 +13,11 @@
 // single spike at 8192).
 //
 // Measured, one fixed-point iteration of a solve with FP64 transforms against these:
-// N = 256 75 -> 56 us, N = 512 213 -> 113 us, N = 1024 755 -> 339 us.  What bounds them now
-// (N = 1024, column pass 297 -> 90 us): integer issue (ALU pipe 47 %, issue 44 %) at 128
-// registers a thread.  Units smaller than a warp (P < 128) keep FP64 butterflies.
+// N = 256 75 -> 56 us, N = 512 213 -> 113 us, N = 1024 755 -> 339 us (column pass 297 -> 90,
+// and 82 us with nothing converted between its transforms).  What bounds them now: latency
+// (barriers, shared memory, twiddle loads) and integer issue.  Tried and slower: twiddles
+// loaded before a stage's barrier (N = 1024 326 -> 335 us), the spectrum column fetched before
+// the last barrier (330).  Units smaller than a warp (P < 128) keep FP64 butterflies.
 //
 //   q in [-2^B, 2^B] at the input of a radix-R butterfly, B = 61 - log2 R: a complex
 //   value then stays below 2^61.5 through the butterfly (|z| grows by R at most).
@@ -226,6 +228,32 @@ __device__ __forceinline__ void fx_store_smem(fx2* buf, int base, const fx2* v, 
     }
 }
 
+// A column of a weight spectrum as the column passes multiply with it: entry k2 holds the
+// halves of w q, w = q 2^(e - 62) with |q| < 2^61 and one exponent e for the column; the low
+// bits of the first 16 real parts hold e + 2^15 (0xffff: the column is not finite); the low bit
+// of every real part is dropped in the product, so a scaled column gives the scaled product.
+__device__ __forceinline__ int fx_spectrum_code(const int4* w, bool valid) {
+    return valid ? (int)(__ballot_sync(0xffffffffu, w[threadIdx.x & 15].y & 1) & 0xffffu) : 1 << 15;
+}
+__device__ __forceinline__ int4 fx_spectrum_entry(double2 w, int k, int k2, int code) {
+    long long re = fx_quantise((unsigned)__double2hiint(w.x), (unsigned)__double2loint(w.x), k);
+    const long long im = fx_quantise((unsigned)__double2hiint(w.y), (unsigned)__double2loint(w.y), k);
+    if (k2 < 16) re = (re & ~1LL) | ((code >> k2) & 1);
+    const FxHalf r = fx_split(re), i = fx_split(im);
+    return make_int4(r.h, r.l, i.h, i.l);
+}
+// Storer of a forward transform that goes on, still in integers, as the inverse transform of
+// its product with a spectrum column, whose outputs `next` takes
+template <class S2> struct FxThen {
+    const int4* w;
+    int code;
+    bool valid;
+    const S2& next;
+    static constexpr bool fx_then = true;
+};
+template <class T, class = void> struct is_fx_then { static constexpr bool value = false; };
+template <class T> struct is_fx_then<T, decltype((void)T::fx_then, void())> { static constexpr bool value = true; };
+
 // the stages with span NS, NS V, ...: integers in buf, exponent E (value = q 2^E)
 template <int DIR, int P, int NS, class S>
 __device__ __forceinline__ void fx_rest(fx2* buf, unsigned* red, int t, const int4* __restrict__ twi, int E, bool bad,
@@ -264,12 +292,36 @@ __device__ __forceinline__ void fx_rest(fx2* buf, unsigned* red, int t, const in
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
         const int k = (t + b * NT) & (NS - 1);
+        if constexpr (NS > 1) {
 #pragma unroll
-        for (int r = 1; r < RAD; ++r) v[b * RAD + r] = fx_cmul<(DIR > 0)>(v[b * RAD + r], __ldg(&twi[k * (r * TWS)]));
+            for (int r = 1; r < RAD; ++r) v[b * RAD + r] = fx_cmul<(DIR > 0)>(v[b * RAD + r], __ldg(&twi[k * (r * TWS)]));
+        }
         fx_dft<DIR, RAD>(&v[b * RAD]);
     }
     __syncthreads();
-    if constexpr (LAST) {
+    if constexpr (LAST && is_fx_then<S>::value) {
+        unsigned o = 0;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const int j = t + b * NT;
+            const int k = j & (NS - 1);
+            const int base = (j - k) * RAD + k;
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) {
+                const int k2 = base + r * NS;
+                int4 w = store.valid ? __ldg(&store.w[k2]) : make_int4(0, 0, 0, 0);
+                w.y &= ~1;                            // (fx_spectrum_code)
+                const fx2 q = fx_cmul<false>(v[b * RAD + r], w);
+                const int hx = (int)(q.x >> 32), hy = (int)(q.y >> 32);
+                o |= (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
+                buf[padi(k2)] = q;
+            }
+        }
+        o = __reduce_or_sync(0xffffffffu, o);
+        if ((t & 31) == 0) red[16 + (t >> 5)] = o;
+        __syncthreads();
+        fx_rest<-DIR, P, 1>(buf, red, t, twi, E + store.code - (1 << 15), bad || store.code == 0xffff, store.next);
+    } else if constexpr (LAST) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             const int j = t + b * NT;
@@ -313,6 +365,24 @@ __device__ __forceinline__ void fx_rest(fx2* buf, unsigned* red, int t, const in
 // lengths whose units are whole warps
 __host__ __device__ constexpr bool fx_length(int P) { return P / fft_values<double>(P) >= 32; }
 
+// the first stage of values v in registers (value = v 2^E), and the rest
+template <int DIR, int P, class S>
+__device__ __forceinline__ void fx_first(fx2* buf, unsigned* red, int t, const int4* __restrict__ twi, fx2* v, int E, bool bad,
+                                         const S& store) {
+    constexpr int V = fft_values<double>(P);
+    fx_dft<DIR, V>(v);
+    unsigned o = 0;
+    auto note = [&](fx2 q) {
+        const int hx = (int)(q.x >> 32), hy = (int)(q.y >> 32);
+        o |= (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
+    };
+    fx_store_smem<P, V, 1>(buf, t * V, v, note);
+    o = __reduce_or_sync(0xffffffffu, o);
+    if ((t & 31) == 0) red[16 + (t >> 5)] = o;
+    __syncthreads();
+    fx_rest<DIR, P, V>(buf, red, t, twi, E, bad, store);
+}
+
 // block_fft in block fixed point (same contract)
 template <int DIR, int P, class L, class S>
 __device__ __forceinline__ void fx_fft(double2* bufd, int t, const double2* __restrict__ tw, const L& load, const S& store) {
@@ -350,17 +420,61 @@ __device__ __forceinline__ void fx_fft(double2* bufd, int t, const double2* __re
         if (!((ZM >> r) & 1u))
             v[r] = fx2{fx_quantise((unsigned)(v[r].x >> 32), (unsigned)v[r].x, k),
                        fx_quantise((unsigned)(v[r].y >> 32), (unsigned)v[r].y, k)};
-    fx_dft<DIR, V>(v);
-    unsigned o = 0;
-    auto note = [&](fx2 q) {
-        const int hx = (int)(q.x >> 32), hy = (int)(q.y >> 32);
-        o |= (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
-    };
-    fx_store_smem<P, V, 1>(buf, t * V, v, note);
-    o = __reduce_or_sync(0xffffffffu, o);
-    if ((t & 31) == 0) red[16 + (t >> 5)] = o;
+    fx_first<DIR, P>(buf, red, t, twi, v, -k, bad, store);
+}
+
+// The transform of the midpoints of P + 2 nodes x[i] = node(i): input j is the cubic midpoint
+// (9 (x[j+1] + x[j+2]) - x[j] - x[j+3]) / 16 for j <= P - 2, and 0 at P - 1.  The nodes are
+// quantised once and the midpoints are integer, at 2^-57 of the largest node; in FP64 they are
+// eight instructions a point, which held the SM longer than the butterflies.  Nodes that
+// are all zero give zero outputs without a transform (the far field of a put above the strike).
+// `node` may read buf.
+template <int DIR, int P, class L, class S>
+__device__ __forceinline__ void fx_fft_mid(double2* bufd, int t, const double2* __restrict__ tw, const L& node, const S& store) {
+    constexpr int V = fft_values<double>(P), NT = P / V, NW = NT / 32;
+    static_assert(NT % 32 == 0 && NW <= 16, "whole warps");
+    fx2* buf = reinterpret_cast<fx2*>(bufd);
+    unsigned* red = fx_slots(bufd, P);
+    const int4* twi = reinterpret_cast<const int4*>(tw + P);
+    fx2 x[V + 1];
+    unsigned big = 0;
+#pragma unroll
+    for (int r = 0; r <= V; ++r) {
+        const double2 d = (r < V || t < 2) ? node(t + r * NT) : make_double2(0.0, 0.0);
+        x[r] = fx2{__double_as_longlong(d.x), __double_as_longlong(d.y)};
+        big = max(big, max((unsigned)(x[r].x >> 32) & 0x7fffffffu, (unsigned)(x[r].y >> 32) & 0x7fffffffu));
+    }
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((t & 31) == 0) red[t >> 5] = big;
+    __syncthreads();                          // also: every node is read before any store
+#pragma unroll
+    for (int u = 0; u < NW; ++u) big = max(big, red[u]);
+    if constexpr (!is_fx_then<S>::value) {
+        if (__syncthreads_or(big != 0) == 0) {
+#pragma unroll
+            for (int r = 0; r < V; ++r) store(t + r * NT, make_double2(0.0, 0.0));
+            __syncthreads();
+            return;
+        }
+    }
+    const bool bad = big >= 0x7ff00000u;
+    const int k = fx_bits(V) - 1 - ((int)(big >> 20) - 1022);
+#pragma unroll
+    for (int r = 0; r <= V; ++r)
+        if (r < V || t < 2)
+            buf[padi(t + r * NT)] = fx2{fx_quantise((unsigned)(x[r].x >> 32), (unsigned)x[r].x, k),
+                                        fx_quantise((unsigned)(x[r].y >> 32), (unsigned)x[r].y, k)};
     __syncthreads();
-    fx_rest<DIR, P, V>(buf, red, t, twi, -k, bad, store);
+    fx2 v[V];
+#pragma unroll
+    for (int r = 0; r < V; ++r) {
+        const int j = t + r * NT;
+        const fx2 a = buf[padi(j)], b = buf[padi(j + 1)], c = buf[padi(j + 2)];
+        const fx2 d = j <= P - 2 ? buf[padi(j + 3)] : fx2{0, 0};
+        v[r] = j <= P - 2 ? fx2{(9 * (b.x + c.x) - (a.x + d.x) + 8) >> 4, (9 * (b.y + c.y) - (a.y + d.y) + 8) >> 4} : fx2{0, 0};
+    }
+    __syncthreads();
+    fx_first<DIR, P>(buf, red, t, twi, v, -k, bad, store);
 }
 // Unscaled length-P complex DFT (DIR = -1: e^{-2 pi i jk/P}, DIR = +1: e^{+...})
 // with input x[j] = load(j) and output X[k] handed to store(k, X[k]);
@@ -373,6 +487,46 @@ __device__ __forceinline__ void block_fft(cpx<R>* buf, int t, const cpx<R>* __re
                                           const S& store) {
     if constexpr (sizeof(R) == 8 && fx_length(P)) fx_fft<DIR, P>(buf, t, tw, load, store);
     else fft_from<R, DIR, P, 1, FUSE2>(buf, t, tw, load, store);
+}
+// A loader marked `mid` gives P + 2 nodes; the transform's inputs are their midpoints.
+template <class T, class = void> struct is_mid { static constexpr bool value = false; };
+template <class T> struct is_mid<T, decltype((void)T::mid, void())> { static constexpr bool value = true; };
+// Forward transform of load(j), product with the spectrum column w (0 where !valid), inverse
+// transform into `store`: the column passes.  In block fixed point the column is in
+// integers (fx_spectrum_entry) and nothing is converted between the transforms: jump sum N = 512 112 -> 96 us, N = 1024
+// 284 -> 250, N = 2048 1019 -> 830, with the integer midpoints of fx_fft_mid.
+template <typename R, int P, class L, class S>
+__device__ __forceinline__ void block_conv(cpx<R>* buf, int t, const cpx<R>* __restrict__ tw, const cpx<R>* w, bool valid,
+                                           const L& load, const S& store) {
+    if constexpr (sizeof(R) == 8 && fx_length(P)) {
+        const int4* wi = reinterpret_cast<const int4*>(w);
+        const FxThen<S> then{wi, fx_spectrum_code(wi, valid), valid, store};
+        if constexpr (is_mid<L>::value) fx_fft_mid<-1, P>(buf, t, tw, load, then);
+        else fx_fft<-1, P>(buf, t, tw, load, then);
+    } else {
+        auto product = [&](int k2, cpx<R> v) { buf[padi(k2)] = cmul(v, valid ? __ldg(&w[k2]) : mk<R>(R(0), R(0))); };
+        if constexpr (is_mid<L>::value) {
+            // nodes staged in buf (constant trip count with a guard: the loop unrolls and its
+            // loads go out together)
+            constexpr int NT = P / fft_values<R>(P);
+#pragma unroll
+            for (int q = 0; q < (P + 2 + NT - 1) / NT; ++q) {
+                const int i = t + q * NT;
+                if (i < P + 2) buf[padi(i)] = load(i);
+            }
+            __syncthreads();
+            auto mid = [&](int i) -> cpx<R> {
+                if (i > P - 2) return mk<R>(R(0), R(0));
+                const cpx<R> x0 = buf[padi(i)], x1 = buf[padi(i + 1)], x2 = buf[padi(i + 2)], x3 = buf[padi(i + 3)];
+                return mk<R>(R(-0.0625) * (x0.x + x3.x) + R(0.5625) * (x1.x + x2.x),
+                             R(-0.0625) * (x0.y + x3.y) + R(0.5625) * (x1.y + x2.y));
+            };
+            block_fft<R, -1, P>(buf, t, tw, mid, product);
+        } else {
+            block_fft<R, -1, P>(buf, t, tw, load, product);
+        }
+        block_fft<R, +1, P>(buf, t, tw, SmemLoad<R>{buf}, store);
+    }
 }
 #endif
 

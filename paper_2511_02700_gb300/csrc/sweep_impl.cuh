@@ -47,7 +47,7 @@ template <typename R, int P> struct Cfg {
     // resident threads per SM: 64 registers a thread in FP32 and in the FP64 transforms of 8 values
     // whose passes fill the chip (P = 2048, 4096: twice the warps outweigh up to 700 bytes of
     // spills in the inverse row pass; jump sum N = 1024 328 -> 284 us, N = 2048 1264 -> 1019 us;
-    // 85 registers at P = 2048: 265 us), 128 otherwise (P = 1024: 114 us against 120 with 64; at
+    // 80 registers at P = 2048: 310 us), 128 otherwise (P = 1024: 114 us against 120 with 64; at
     // P = 8192 16 values a thread spill, its row pass takes 674 us against 497)
     static constexpr int TPS = sizeof(R) == 4 || P == 2048 || P == 4096 ? 1024 : 512;
     static constexpr int MINB = TPS / THREADS < 24 ? TPS / THREADS : 24;
@@ -294,11 +294,15 @@ __device__ __forceinline__ void row_forward_body(const FwdArgs<R>& a, int upb) {
             }
         }
         __syncthreads();
-        auto load = [&](int i) -> C {
-            if (i > P - 2) return mk<R>(0, 0);
-            return mk<R>(midpoint(nodes, i), midpoint(nodes + P + 2, i));
-        };
-        block_fft<R, -1, P>(buf, t, tw, load, SmemStore<R>{buf});
+        if constexpr (sizeof(R) == 8 && fx_length(P)) {
+            fx_fft_mid<-1, P>(buf, t, tw, [&](int i) { return make_double2(nodes[i], nodes[P + 2 + i]); }, SmemStore<R>{buf});
+        } else {
+            auto load = [&](int i) -> C {
+                if (i > P - 2) return mk<R>(0, 0);
+                return mk<R>(midpoint(nodes, i), midpoint(nodes + P + 2, i));
+            };
+            block_fft<R, -1, P>(buf, t, tw, load, SmemStore<R>{buf});
+        }
     }
     store_spectrum_rows<R, P>(buf, (C*)a.S, a.g.rows, a.g.ng, rho, t, valid);
 }
@@ -326,6 +330,18 @@ __host__ __device__ constexpr unsigned incr_zero_mask() {
 template <typename R, int P>
 struct IncrColLoad {
     static constexpr unsigned zero_mask = incr_zero_mask<R, P>();
+    const cpx<R>* col;
+    int rlo, rhi;
+    bool valid;
+    __device__ __forceinline__ cpx<R> operator()(int rho) const {
+        return (valid && rho >= rlo && rho < rhi) ? col[(size_t)rho * cgroup<R>()] : mk<R>(0, 0);
+    }
+};
+
+// nodes of a full column, rows rlo..rhi-1 of the column group (zero elsewhere)
+template <typename R>
+struct FullColLoad {
+    static constexpr bool mid = true;
     const cpx<R>* col;
     int rlo, rhi;
     bool valid;
@@ -364,35 +380,13 @@ __device__ __forceinline__ void col_body(const ColArgs<R>& a, int upb) {
             l2_prefetch((const C*)a.S + ((size_t)gn * a.g.rows + r0) * Gc, (size_t)(r1 - r0) * Gc * sizeof(C));
         }
     }
-    auto store_mul = [&](int k2, C v) {
-        const C w = valid ? __ldg(&wh[k2]) : mk<R>(0, 0);
-        buf[padi(k2)] = cmul(v, w);
-    };
-    if constexpr (INCR) {
-        // raw rows; the midpoint interpolation along s2 is in the weight spectrum.
-        // Rows outside [N/2 + 2, 3N/2 + 2) are zero
-        block_fft<R, -1, P>(buf, t, tw, IncrColLoad<R, P>{col, a.rlo, a.rhi, valid}, store_mul);
-    } else {
-        // (constant trip count with a guard: the loop unrolls and its loads go out together)
-#pragma unroll
-        for (int q = 0; q < (P + 2 + NT - 1) / NT; ++q) {
-            const int rho = t + q * NT;
-            if (rho < P + 2)
-                buf[padi(rho)] = (valid && rho >= a.rlo && rho < a.rhi) ? col[(size_t)rho * Gc] : mk<R>(0, 0);
-        }
-        __syncthreads();
-        auto load = [&](int i) -> C {
-            if (i > P - 2) return mk<R>(0, 0);
-            const C x0 = buf[padi(i)], x1 = buf[padi(i + 1)], x2 = buf[padi(i + 2)], x3 = buf[padi(i + 3)];
-            return mk<R>(R(-0.0625) * (x0.x + x3.x) + R(0.5625) * (x1.x + x2.x),
-                         R(-0.0625) * (x0.y + x3.y) + R(0.5625) * (x1.y + x2.y));
-        };
-        block_fft<R, -1, P>(buf, t, tw, load, store_mul);
-    }
     auto store_out = [&](int m, C v) {
         if (valid && m >= 1 && m <= N) col[(size_t)(m - 1) * Gc] = v;
     };
-    block_fft<R, +1, P>(buf, t, tw, SmemLoad<R>{buf}, store_out);
+    // INCR: raw rows; the midpoint interpolation along s2 is in the weight spectrum.
+    // Rows outside [N/2 + 2, 3N/2 + 2) are zero
+    if constexpr (INCR) block_conv<R, P>(buf, t, tw, wh, valid, IncrColLoad<R, P>{col, a.rlo, a.rhi, valid}, store_out);
+    else block_conv<R, P>(buf, t, tw, wh, valid, FullColLoad<R>{col, a.rlo, a.rhi, valid}, store_out);
 }
 template <typename R, int P, bool INCR>
 PIDE_FFT_KERNEL(R, P) k_col(const __grid_constant__ ColArgs<R> a) { col_body<R, P, INCR>(a, Cfg<R, P>::UNITS); }
@@ -1841,12 +1835,7 @@ PIDE_FFT_KERNEL(R, P) k_ps_col(void* Sv, const void* Whv, PsInterp ip, const voi
         }
         return mk<R>(x.value(), y.value());
     };
-    auto store_mul = [&](int k2, C v) {
-        const C w = valid ? __ldg(&wh[k2]) : mk<R>(0, 0);
-        buf[padi(k2)] = cmul(v, w);
-    };
-    block_fft<R, -1, P>(buf, t, tw, load, store_mul);
-    block_fft<R, +1, P>(buf, t, tw, SmemLoad<R>{buf}, SmemStore<R>{buf});
+    block_conv<R, P>(buf, t, tw, wh, valid, load, SmemStore<R>{buf});
     for (int m = t; m < ip.rows && valid; m += NT) {
         TapSum<R> x, y;
         if (m < ip.n1) {
@@ -1939,17 +1928,57 @@ PIDE_FFT_KERNEL(double, P) k_weights_col(Geometry g, const double2* Sd, cpx<RO>*
                           0.5625 * a1.y + 0.5625 * a2.y - 0.0625 * a3.y);
     };
     const double2 c1 = valid ? chat(k1) : mk<double>(0, 0);
+    auto incr = [&](int k2, double2 w) { return cmul(cmul(w, c1), chat(k2)); };
     // column-major: column k1 at k1 P, contiguous for the column pass that reads it
-    auto store = [&](int k2, double2 w) {
-        if (!valid) return;
-        const size_t o = (size_t)k1 * P + k2;
-        Wh[o] = mk<RO>((RO)(w.x * inv), (RO)(-w.y * inv));
-        if (Whi) {
-            const double2 wc = cmul(cmul(w, c1), chat(k2));
-            Whi[o] = mk<RO>((RO)(wc.x * inv), (RO)(-wc.y * inv));
+    if constexpr (sizeof(RO) == 8 && fx_length(P)) {
+        // in integers (fx_spectrum_entry): each column's largest magnitude first
+        __shared__ unsigned red[2][CF::THREADS / 32];
+        block_fft<double, -1, P>(buf, t, twd, load, SmemStore<double>{buf});
+        unsigned big[2] = {0, 0};
+        auto note = [](unsigned m, double2 v) {
+            return max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+        };
+        for (int k2 = t; k2 < P; k2 += NT) {
+            const double2 w = buf[padi(k2)];
+            big[0] = note(big[0], w);
+            if (Whi) big[1] = note(big[1], incr(k2, w));
         }
-    };
-    block_fft<double, -1, P>(buf, t, twd, load, store);
+        int k[2], code[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const unsigned m = __reduce_max_sync(0xffffffffu, big[i]);
+            if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = m;
+        }
+        __syncthreads();
+        if (!valid) return;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            unsigned m = 0;
+            for (int u = 0; u < NT / 32; ++u) m = max(m, red[i][unit * (NT / 32) + u]);
+            k[i] = 61 - ((int)(m >> 20) - 1022);
+            code[i] = m >= 0x7ff00000u ? 0xffff : 62 - k[i] - 2 * log2_t<P>::value + (1 << 15);     // the factor 1/P^2
+        }
+        for (int k2 = t; k2 < P; k2 += NT) {
+            const double2 w = buf[padi(k2)];
+            const size_t o = (size_t)k1 * P + k2;
+            reinterpret_cast<int4*>(Wh)[o] = fx_spectrum_entry(mk<double>(w.x, -w.y), k[0], k2, code[0]);
+            if (Whi) {
+                const double2 wc = incr(k2, w);
+                reinterpret_cast<int4*>(Whi)[o] = fx_spectrum_entry(mk<double>(wc.x, -wc.y), k[1], k2, code[1]);
+            }
+        }
+    } else {
+        auto store = [&](int k2, double2 w) {
+            if (!valid) return;
+            const size_t o = (size_t)k1 * P + k2;
+            Wh[o] = mk<RO>((RO)(w.x * inv), (RO)(-w.y * inv));
+            if (Whi) {
+                const double2 wc = incr(k2, w);
+                Whi[o] = mk<RO>((RO)(wc.x * inv), (RO)(-wc.y * inv));
+            }
+        };
+        block_fft<double, -1, P>(buf, t, twd, load, store);
+    }
 }
 
 // ---------------------------------------------------------------------------
