@@ -56,6 +56,7 @@ void gauss_legendre(int n, double* x, double* w) {
 constexpr int kGlNear = 10, kGlFar = 6, kGlEdge = 32, kGlPay = 16, kGlVfar = 4;
 constexpr double kTanhSinhStep = 0.125;
 constexpr int kGlTotal = 2 * (kGlNear + kGlFar + kGlEdge + kGlPay + kGlVfar);
+constexpr int kKpolyOff = (kGlTotal + kKtabMax + 1) / 2 * 2;       // 16-byte aligned
 
 enum Region {
     R_V0, R_V1, R_V2, R_V3, R_V4, R_BV, R_BY, R_W, R_X, R_OUT,   // 10 state-sized fields
@@ -101,10 +102,10 @@ void fill_layout(int N, Layout& L) {
     L.size[R_SIN2D] = (size_t)(N + 1) * 8;
     L.size[R_SIN2R] = (size_t)(N + 1) * sizeof(R);
     L.size[R_OMEGA] = (size_t)N * N * 8;
-    L.size[R_PART] = (size_t)((N * N + 255) / 256) * 3 * 8;
+    L.size[R_PART] = weights_blocks(N) * 3 * 8;
     L.size[R_PARAMS] = 16 * 8;
     L.size[R_MOMENT] = moment_doubles() * 8;
-    L.size[R_GL] = (size_t)(kGlTotal + kKtabMax) * 8;     // quadrature nodes, then the K_nu table
+    L.size[R_GL] = (size_t)(kKpolyOff + 8 * kKtabMax) * 8;     // quadrature nodes, the K_nu table, its polynomials
     L.size[R_RESID] = 16;
     L.size[R_CTL] = sizeof(FpCtl);
     size_t o = 0;
@@ -929,9 +930,12 @@ static cudaError_t precompute_core(int N, double hz, double* dgl, const pide2d_m
         // the adjoint's central differences) read the same interpolant of x
         const double u0 = du * std::floor(std::log(x_lo) / du - 5.0);
         double* tab = dgl + kGlTotal;
-        const cudaError_t te = launch_ktab(L.nu, u0, du, n, tab, s);
+        double* poly = dgl + kKpolyOff;
+        const cudaError_t te = launch_ktab(L.nu, u0, du, n, tab, poly, s);
         if (te != cudaSuccess) return te;
         L.ktab = tab;
+        L.kpoly = poly;
+        L.logc1 = std::log(L.c1);
         L.ku0 = u0;
         L.kidu = 1.0 / du;
         L.kn = n;
@@ -2195,10 +2199,10 @@ void price_layout(pide2d_price* H) {
         o += align256(bytes);
         return at;
     };
-    H->off_gl = take((size_t)(kGlTotal + kKtabMax) * 8);
+    H->off_gl = take((size_t)(kKpolyOff + 8 * kKtabMax) * 8);
     H->off_omega = take((size_t)nzz * nzz * 8);
     H->off_pad = take((size_t)(P / 2) * (P / 2) * 8);
-    H->off_part = take((size_t)((nzz * nzz + 255) / 256) * 3 * 8);
+    H->off_part = take(weights_blocks(nzz) * 3 * 8);
     H->off_moment = take(moment_doubles() * 8);
     H->off_params = take(16 * 8);
     H->off_rows = take((size_t)spectrum_groups<double>(P) * P * cgroup_bytes<double>());

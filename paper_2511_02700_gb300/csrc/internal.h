@@ -354,11 +354,12 @@ struct LevyParams {
     double gamma_nu;         // Gamma(nu)
     // ln(e^x K_nu(x)) at u = ku0 + i / kidu, i < kn (NULL: no table)
     const double* ktab;
-    double ku0, kidu;
+    const double* kpoly;     // 8 polynomial coefficients for each interval of the table
+    double ku0, kidu, logc1; // logc1 = ln c1
     int kn;
 };
-constexpr int kKtabMax = 4096;          // entries of the K_nu table (after the quadrature nodes)
-cudaError_t launch_ktab(double nu, double u0, double du, int n, double* tab, cudaStream_t s);
+constexpr int kKtabMax = 4096;          // entries of the K_nu table (after the quadrature nodes; its polynomials follow)
+cudaError_t launch_ktab(double nu, double u0, double du, int n, double* tab, double* poly, cudaStream_t s);
 struct WeightJob {
     int N;
     double h;
@@ -367,6 +368,11 @@ struct WeightJob {
     const double* gl_far_x; const double* gl_far_w; int n_far;
     const double* gl_vfar_x; const double* gl_vfar_w; int n_vfar;
 };
+// rows of cells a thread of k_weights takes, and its blocks (three partial sums each)
+constexpr int weights_rows(int N) { return N >= 2048 ? 4 : 1; }
+constexpr size_t weights_blocks(int N) {
+    return (size_t)((N + 31) / 32) * ((N + 8 * weights_rows(N) - 1) / (8 * weights_rows(N)));
+}
 cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, double* omega, double* partials,
                            int* nblocks, cudaStream_t s);
 // the R_I moment (eq. 3.3): blocks of the quadrature and the doubles of its buffer

@@ -40,48 +40,69 @@ __device__ double bessel_k_scaled(double nu, double x) {
 }
 
 
-// ln(e^x K_nu(x)): 8-point Lagrange interpolation in u = ln x on the
+// ln(e^x K_nu(x)) at x = e^u: 8-point Lagrange interpolation in u on the
 // model's table (nodes base..base+7 around u), else the trapezoidal sum.  In u
 // the function is smooth (slope -nu for small x, -1/2 for large x); at a node
 // spacing of 0.01 the interpolation error is below 1e-14 absolute, the
-// rounding level of the sum it replaces.
-__device__ double log_ek(const LevyParams& L, double x) {
+// rounding level of the sum it replaces.  Each interval's interpolant is kept as
+// a polynomial about its middle (k_kpoly): 8 FP64 instructions where the Lagrange
+// form took 45.
+__device__ double log_ek(const LevyParams& L, double u) {
     if (L.ktab) {
-        const double f = (log(x) - L.ku0) * L.kidu;
+        const double f = (u - L.ku0) * L.kidu;
         const int base = (int)floor(f) - 3;
         if (base >= 0 && base + 7 < L.kn) {
-            const double t = f - (double)base;             // in [3, 4)
-            // l_a(t) = prod_{b != a} (t - b) / (a - b) = pre_a suf_a c_a
-            constexpr double c[8] = {-1.0 / 5040.0, 1.0 / 720.0, -1.0 / 240.0, 1.0 / 144.0,
-                                     -1.0 / 144.0,  1.0 / 240.0, -1.0 / 720.0, 1.0 / 5040.0};
-            double pre[8], suf[8];
-            pre[0] = 1.0;
-#pragma unroll
-            for (int a = 1; a < 8; ++a) pre[a] = pre[a - 1] * (t - (double)(a - 1));
-            suf[7] = 1.0;
-#pragma unroll
-            for (int a = 6; a >= 0; --a) suf[a] = suf[a + 1] * (t - (double)(a + 1));
-            const double* T = L.ktab + base;
-            double v = 0.0;
-#pragma unroll
-            for (int a = 0; a < 8; ++a) v += (pre[a] * suf[a] * c[a]) * T[a];
-            return v;
+            const double t = f - ((double)base + 3.5);         // in [-1/2, 1/2)
+            const double2* c = reinterpret_cast<const double2*>(L.kpoly + 8 * (size_t)base);
+            const double2 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2), c67 = __ldg(c + 3);
+            return c01.x + t * (c01.y + t * (c23.x + t * (c23.y + t * (c45.x + t * (c45.y + t * (c67.x + t * c67.y))))));
         }
     }
-    return log(bessel_k_scaled(L.nu, x));
+    return log(bessel_k_scaled(L.nu, exp(u)));
+}
+
+// the interpolating polynomial of table entries i .. i + 7 in t, entry i + a at t = a - 7/2
+__global__ void k_kpoly(const double* __restrict__ tab, int n, double* __restrict__ poly) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i + 7 >= n) return;
+    // coefficient of t^j of the Lagrange basis polynomial a < 4; that of 7 - a has the sign (-1)^j
+    constexpr double m[8][4] = {
+            {-5.0 / 2048.0, 49.0 / 2048.0, -245.0 / 2048.0, 1225.0 / 2048.0},
+            {5.0 / 7168.0, -49.0 / 5120.0, 245.0 / 3072.0, -1225.0 / 1024.0},
+            {259.0 / 23040.0, -499.0 / 4608.0, 1299.0 / 2560.0, -1891.0 / 4608.0},
+            {-37.0 / 11520.0, 499.0 / 11520.0, -433.0 / 1280.0, 1891.0 / 2304.0},
+            {-7.0 / 1152.0, 59.0 / 1152.0, -15.0 / 128.0, 83.0 / 1152.0},
+            {1.0 / 576.0, -59.0 / 2880.0, 5.0 / 64.0, -83.0 / 576.0},
+            {1.0 / 1440.0, -1.0 / 288.0, 1.0 / 160.0, -1.0 / 288.0},
+            {-1.0 / 5040.0, 1.0 / 720.0, -1.0 / 240.0, 1.0 / 144.0}};
+    double e[4], o[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        e[a] = tab[i + a] + tab[i + 7 - a];
+        o[a] = tab[i + a] - tab[i + 7 - a];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        double c = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) c += m[j][a] * (j % 2 ? o[a] : e[a]);
+        poly[8 * (size_t)i + j] = c;
+    }
 }
 
 // x^nu K_nu(x), bounded as x -> 0 (limit 2^(nu-1) Gamma(nu))
 __device__ double xnu_knu(const LevyParams& L, double x) {
     if (x < 1e-8) return exp2(L.nu - 1.0) * L.gamma_nu;
-    return exp(L.nu * log(x) - x + log_ek(L, x));
+    const double u = log(x);
+    return exp(L.nu * u - x + log_ek(L, u));
 }
 
 // l(z), Sec. 4
 __device__ double levy_density(const LevyParams& L, double z1, double z2) {
-    const double zn = sqrt(L.Ri11 * z1 * z1 + 2.0 * L.Ri12 * z1 * z2 + L.Ri22 * z2 * z2);
-    const double x = L.c1 * zn;
-    return exp(L.logpref + log_ek(L, x) - x - L.nu * log(zn) + L.b1 * z1 + L.b2 * z2);
+    // one logarithm serves K_nu's table and |z|^-nu
+    const double q = L.Ri11 * z1 * z1 + 2.0 * L.Ri12 * z1 * z2 + L.Ri22 * z2 * z2;
+    const double lz = 0.5 * log(q);
+    return exp(L.logpref + log_ek(L, lz + L.logc1) - L.c1 * sqrt(q) - L.nu * lz + L.b1 * z1 + L.b2 * z2);
 }
 
 // the table of log_ek: ln(e^x K_nu(x)) at x = e^{u0 + i du}, i < n.  One warp per
@@ -107,10 +128,14 @@ __global__ void k_ktab(double nu, double u0, double du, int n, double* tab) {
     if (lane == 0) tab[i] = log((0.5 + s) * h);
 }
 
-// R_II cells up to this ||z_l||_inf / h (the 10-point rule, 100 nodes) take a
-// warp each (k_weights_near); the cells beyond, with 36 or 16 nodes, are
-// numerous enough to fill the GPU one thread per cell, at full lane use
-__host__ __device__ __forceinline__ int weights_warp_zone(const WeightJob& j) { return j.M2 < 8 ? j.M2 : 8; }
+// R_II cells up to this ||z_l||_inf / h take a warp each (k_weights_near): those of the
+// 10-point rule (100 nodes), and on lattices up to 256 all of them, where a thread's 36
+// nodes in turn took longer than everything else (N = 128: 256 us for all
+// weights, 56 so; N = 1024 942 -> 567, N = 4096 13.2 -> 6.9 ms by the cheaper density).  Beyond, the cells are
+// numerous enough to fill the GPU one thread per cell, at full lane use.
+__host__ __device__ __forceinline__ int weights_warp_zone(const WeightJob& j) {
+    return j.M2 < 8 || j.N <= 256 ? j.M2 : 8;
+}
 
 // the R_II cell integral at node (a, b) of its product rule (eq. 3.5 with the
 // |z|^2 factor of the modified midpoint rule)
@@ -134,9 +159,10 @@ __global__ void k_weights_near(LevyParams L, WeightJob j, double* omega) {
     const int l1 = q1 - Z, l2 = q2 - Z;               // cells l = -Z .. Z - 1 around the origin
     const double inf = fmax(fabs(l1 + 0.5), fabs(l2 + 0.5));
     if (inf <= 2.0 || inf > (double)Z) return;
-    const int n = j.n_near;                           // inf <= 8: the 10-point rule
-    const double* gx = j.gl_near_x;
-    const double* gw = j.gl_near_w;
+    const bool near = inf <= 8.0;                     // (the rules of k_weights; its 4-point one starts at N = 1024)
+    const int n = near ? j.n_near : j.n_far;
+    const double* gx = near ? j.gl_near_x : j.gl_far_x;
+    const double* gw = near ? j.gl_near_w : j.gl_far_w;
     const double c1 = (l1 + 0.5) * j.h, c2 = (l2 + 0.5) * j.h;
     double acc = 0.0;
     for (int k = lane; k < n * n; k += 32) acc += rii_node(L, c1, c2, j.h, gx, gw, k / n, k - (k / n) * n);
@@ -152,12 +178,20 @@ __global__ void k_weights_near(LevyParams L, WeightJob j, double* omega) {
 // weights, eq. 3.5; one thread per cell, per-block partial sums of
 // (w, w (e^{z1} - 1), w (e^{z2} - 1)) for the deterministic final reduction
 // ---------------------------------------------------------------------------
-__global__ void k_weights(LevyParams L, WeightJob j, double* omega, double* partials) {
+__global__ void k_weights(LevyParams L, WeightJob j, int rows, double* omega, double* partials) {
+    // 32 x 8 threads; a thread takes `rows` cells of its column, which share expm1(c1)
     const int N = j.N;
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    double w = 0.0, e1 = 0.0, e2 = 0.0;
-    if (cell < N * N) {
-        const int i2 = cell / N, i1 = cell - i2 * N;
+    const int i1 = blockIdx.x * 32 + threadIdx.x, lane = threadIdx.y * 32 + threadIdx.x;
+    __shared__ double m2[32];
+    if (lane < 8 * rows) m2[lane] = expm1(((int)(blockIdx.y * 8 * rows) + lane - N / 2 + 0.5) * j.h);
+    __syncthreads();
+    const double m1 = expm1((i1 - N / 2 + 0.5) * j.h);
+    double w0 = 0.0, e1 = 0.0, e2 = 0.0;
+    for (int r = 0; r < rows; ++r) {
+        const int row = threadIdx.y + 8 * r, i2 = blockIdx.y * 8 * rows + row;
+        if (i1 >= N || i2 >= N) break;
+        const size_t cell = (size_t)i2 * N + i1;
+        double w = 0.0;
         const int l1 = i1 - N / 2, l2 = i2 - N / 2;
         const double c1 = (l1 + 0.5) * j.h, c2 = (l2 + 0.5) * j.h;
         const double inf = fmax(fabs(l1 + 0.5), fabs(l2 + 0.5));   // ||z_l||_inf / h
@@ -189,26 +223,28 @@ __global__ void k_weights(LevyParams L, WeightJob j, double* omega, double* part
             w = levy_density(L, c1, c2) * j.h * j.h;
         }
         omega[cell] = w;
-        e1 = w * expm1(c1);
-        e2 = w * expm1(c2);
+        w0 += w;
+        e1 += w * m1;
+        e2 += w * m2[row];
     }
     __shared__ double sw[256], s1[256], s2[256];
-    sw[threadIdx.x] = w;
-    s1[threadIdx.x] = e1;
-    s2[threadIdx.x] = e2;
+    sw[lane] = w0;
+    s1[lane] = e1;
+    s2[lane] = e2;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            sw[threadIdx.x] += sw[threadIdx.x + o];
-            s1[threadIdx.x] += s1[threadIdx.x + o];
-            s2[threadIdx.x] += s2[threadIdx.x + o];
+    for (int o = 128; o > 0; o >>= 1) {
+        if (lane < o) {
+            sw[lane] += sw[lane + o];
+            s1[lane] += s1[lane + o];
+            s2[lane] += s2[lane + o];
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x + 0] = sw[0];
-        partials[3 * blockIdx.x + 1] = s1[0];
-        partials[3 * blockIdx.x + 2] = s2[0];
+    if (lane == 0) {
+        const size_t b = blockIdx.y * (size_t)gridDim.x + blockIdx.x;
+        partials[3 * b + 0] = sw[0];
+        partials[3 * b + 1] = s1[0];
+        partials[3 * b + 2] = s2[0];
     }
 }
 
@@ -481,14 +517,15 @@ __global__ void k_ring(Geometry g, const double* E1d, const double* E2d, double 
 // ---------------------------------------------------------------------------
 cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, double* omega, double* partials, int* nblocks,
                            cudaStream_t s) {
-    const int cells = j.N * j.N;
-    const int nb = (cells + 255) / 256;
-    *nblocks = nb;
+    // four rows a thread save exponentials and partial sums where the cells fill the chip
+    const int rows = weights_rows(j.N);
+    *nblocks = (int)weights_blocks(j.N);
+    const dim3 grd((j.N + 31) / 32, *nblocks / ((j.N + 31) / 32));
     const int side = 2 * weights_warp_zone(j);
     k_weights_near<<<(side * side + 7) / 8, 256, 0, s>>>(L, j, omega);       // eight cells per block
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_weights<<<nb, 256, 0, s>>>(L, j, omega, partials);
+    k_weights<<<grd, dim3(32, 8), 0, s>>>(L, j, rows, omega, partials);
     return cudaGetLastError();
 }
 cudaError_t launch_moment(const LevyParams& L, double H, const double* glx, const double* glw, int ngl, double tsh,
@@ -506,8 +543,11 @@ cudaError_t launch_finalize(const double* partials, int nblocks, const double* m
     k_finalize<<<1, 1024, 0, s>>>(partials, nblocks, moment, r, sigma_cov[0], sigma_cov[1], sigma_cov[2], params);
     return cudaGetLastError();
 }
-cudaError_t launch_ktab(double nu, double u0, double du, int n, double* tab, cudaStream_t s) {
+cudaError_t launch_ktab(double nu, double u0, double du, int n, double* tab, double* poly, cudaStream_t s) {
     k_ktab<<<(n + 3) / 4, 128, 0, s>>>(nu, u0, du, n, tab);      // four entries per block
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_kpoly<<<(n + 127) / 128, 128, 0, s>>>(tab, n, poly);
     return cudaGetLastError();
 }
 cudaError_t launch_tables(int N, double s_lo1, double s_lo2, double h, double* E1d, double* E2d, float* E1f,
