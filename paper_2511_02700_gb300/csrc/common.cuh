@@ -28,6 +28,20 @@ template <typename R> using cpx = typename cpx_t<R>::type;
 template <typename R> __device__ __forceinline__ cpx<R> mk(R x, R y) { cpx<R> c; c.x = x; c.y = y; return c; }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { a.x += b.x; a.y += b.y; return a; }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { a.x -= b.x; a.y -= b.y; return a; }
+// FP32 pairs by the packed instructions, one issue slot instead of two (the passes are bound by
+// issue and latency): 64 steps at N = 4096 207.4 -> 205.4 ms, N = 512 jump sum 81 -> 79 us
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+    float2 r;
+    asm("{.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 s, p, q;\n\tmov.b64 {%0, %1}, s;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+    float2 r;
+    asm("{.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tsub.rn.f32x2 s, p, q;\n\tmov.b64 {%0, %1}, s;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
     C c; c.x = a.x * b.x - a.y * b.y; c.y = a.x * b.y + a.y * b.x; return c;
 }
@@ -165,8 +179,16 @@ __device__ __forceinline__ void dit_bfly(C* v) {
         if constexpr (K < LEN / 2) {
             C a = v[I + K];
             C b = mul_w16<DIR, K*(16 / LEN)>(v[I + K + LEN / 2]);
-            v[I + K] = cadd(a, b);
-            v[I + K + LEN / 2] = csub(a, b);
+            if constexpr (K * (16 / LEN) % 16 == 4) {
+                // a rotation by i is free in scalar instructions (register choice and sign)
+                v[I + K].x = a.x + b.x;
+                v[I + K].y = a.y + b.y;
+                v[I + K + LEN / 2].x = a.x - b.x;
+                v[I + K + LEN / 2].y = a.y - b.y;
+            } else {
+                v[I + K] = cadd(a, b);
+                v[I + K + LEN / 2] = csub(a, b);
+            }
             dit_bfly<DIR, RAD, LEN, I, K + 1>(v);
         } else {
             dit_bfly<DIR, RAD, LEN, I + LEN, 0>(v);
