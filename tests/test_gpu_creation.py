@@ -38,7 +38,8 @@ def test_weight_samples_and_rates(n):
     c = (np.arange(-(n // 2), n // 2) + 0.5) * g.h
     rng = np.random.Generator(np.random.PCG64(n))
     i2, i1 = rng.integers(0, n, (2, 400))
-    outer = np.maximum(np.abs(c[i1]), np.abs(c[i2])) > np.ceil(np.sqrt(0.1) * (n // 2) - 0.5) * g.h
+    # cells weighted by the density at their centre: beyond the zero weights and the integrated cells
+    outer = np.maximum(np.abs(c[i1]), np.abs(c[i2])) > max(2.0, np.ceil(np.sqrt(0.1) * (n // 2) - 0.5)) * g.h
     want = levy_density(m, c[i1[outer]], c[i2[outer]]) * g.h ** 2
     assert outer.any() and np.abs(om[i2[outer], i1[outer]] / want - 1.0).max() < 1e-11
     inf = np.maximum(np.abs(c)[None, :], np.abs(c)[:, None]) / g.h
