@@ -261,7 +261,8 @@ cudaError_t launch_ps_bicg(const PsBicgArgs& a, int blocks, cudaStream_t s);
 cudaError_t launch_ps_update(size_t n, const double* X, double* Y, double* T, double* part, double* res, cudaStream_t s);
 cudaError_t launch_ps_sl(int n1, const int* s1, const double* w1, const int* s2, const double* w2, const double* Z,
                          double* W, cudaStream_t s);
-// omega-hat: forward column FFT of the FP64 row spectra, written as cpx<RO>
+// omega-hat: forward column FFT of the FP64 row spectra, written as cpx<RO>, or for RO = double and P >= 128 as
+// integer columns (fx_spectrum_entry in fixfft.cuh)
 template <typename RO> cudaError_t launch_weights_col(const Geometry& g, const void* Sd, void* Wh, void* Whi,
                                                        const void* twd, cudaStream_t s);
 template <typename R> cudaError_t launch_state_from_double(const Geometry& g, const double* src, int ld_src,
