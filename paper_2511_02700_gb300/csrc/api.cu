@@ -258,7 +258,7 @@ TapeLayout tape_layout(const Layout& L, int n_steps, int interval, int ndirs) {
     t.field = align256(L.size[R_V0]);
     t.spec1 = align256(L.size[R_WH]);
     t.omega = align256((size_t)N * N * 8);
-    t.part = align256(L.size[R_PART]);
+    t.part = align256(gradient_weights_blocks(N) * 3 * 8);
     t.rows = align256((size_t)spectrum_groups<double>(L.g.P) * L.g.P * cgroup_bytes<double>());
     t.nparts = align256((size_t)adjoint_dot_blocks(N) * 4 * 8);
     t.nckpt = (n_steps + interval - 1) / interval;
@@ -892,8 +892,9 @@ static std::vector<double> quadrature_nodes() {
     return gl;
 }
 
-// the precompute on a z-lattice of N x N cells of width hz (N_z = N/2)
-static cudaError_t precompute_core(int N, double hz, double* dgl, const pide2d_model& m, double* omega,
+// the precompute on a z-lattice of N x N cells of width hz (N_z = N/2); `gradient`: in the form
+// whose differences over models the adjoint takes (part: gradient_weights_blocks)
+static cudaError_t precompute_core(int N, double hz, double* dgl, const pide2d_model& m, bool gradient, double* omega,
                                    double* part, double* moment, double* params, cudaStream_t s) {
     // Levy density constants (Sec. 4)
     const double r11 = m.rho[0], r12 = m.rho[1], r22 = m.rho[2];
@@ -931,7 +932,7 @@ static cudaError_t precompute_core(int N, double hz, double* dgl, const pide2d_m
         const double u0 = du * std::floor(std::log(x_lo) / du - 5.0);
         double* tab = dgl + kGlTotal;
         double* poly = dgl + kKpolyOff;
-        const cudaError_t te = launch_ktab(L.nu, u0, du, n, tab, poly, s);
+        const cudaError_t te = launch_ktab(L.nu, u0, du, n, tab, gradient ? nullptr : poly, s);
         if (te != cudaSuccess) return te;
         L.ktab = tab;
         L.kpoly = poly;
@@ -955,19 +956,19 @@ static cudaError_t precompute_core(int N, double hz, double* dgl, const pide2d_m
     j.gl_vfar_w = j.gl_vfar_x + kGlVfar;
     j.n_vfar = kGlVfar;
     int nblocks = 0;
-    cudaError_t e = launch_weights(L, j, omega, part, &nblocks, s);
+    cudaError_t e = launch_weights(L, j, gradient, omega, part, &nblocks, s);
     if (e != cudaSuccess) return e;
     const double* edge = dgl + 2 * (kGlNear + kGlFar);
-    e = launch_moment(L, 2.0 * hz, edge, edge + kGlEdge, kGlEdge, kTanhSinhStep, moment, s);
+    e = launch_moment(L, gradient, 2.0 * hz, edge, edge + kGlEdge, kGlEdge, kTanhSinhStep, moment, s);
     if (e != cudaSuccess) return e;
     return launch_finalize(part, nblocks, moment, m.r, m.sigma_cov, params, s);
 }
 
 // weights w (eq. 3.5), the R_I moment (eq. 3.3) and the rates (eq. 3.6) of a
 // model, into the given device buffers (params: the 9 values of pide2d_get_weights)
-static pide2d_status run_precompute(pide2d* H, const pide2d_model& m, double* omega, double* part, double* moment,
-                                    double* params) {
-    PIDE_CUDA(precompute_core(H->L.g.N, H->h, H->at<double>(R_GL), m, omega, part, moment, params, H->stream));
+static pide2d_status run_precompute(pide2d* H, const pide2d_model& m, bool gradient, double* omega, double* part,
+                                    double* moment, double* params) {
+    PIDE_CUDA(precompute_core(H->L.g.N, H->h, H->at<double>(R_GL), m, gradient, omega, part, moment, params, H->stream));
     return PIDE2D_OK;
 }
 
@@ -1102,7 +1103,7 @@ static pide2d_status do_create(pide2d* H) {
     // omega-hat = conj(fft2(Omega padded))/P^2 (eq. 3.13) with the FP64 row
     // spectra in the (not yet used) state-field region
     {
-        const pide2d_status ps = run_precompute(H, H->model, H->at<double>(R_OMEGA), H->at<double>(R_PART),
+        const pide2d_status ps = run_precompute(H, H->model, false, H->at<double>(R_OMEGA), H->at<double>(R_PART),
                                                 H->at<double>(R_MOMENT), H->at<double>(R_PARAMS));
         if (ps != PIDE2D_OK) return ps;
     }
@@ -1944,9 +1945,9 @@ static pide2d_status do_adjoint(pide2d* H, const pide2d_model* dirs, int ndirs, 
         mp.lambda += eps * d.lambda;         mm.lambda -= eps * d.lambda;
         for (int i = 0; i < 2; ++i) { mp.eta[i] += eps * d.eta[i]; mm.eta[i] -= eps * d.eta[i]; }
         for (int i = 0; i < 3; ++i) { mp.rho[i] += eps * d.rho[i]; mm.rho[i] -= eps * d.rho[i]; }
-        pide2d_status ps = run_precompute(H, mp, om_p, part, moment, par_p);
+        pide2d_status ps = run_precompute(H, mp, true, om_p, part, moment, par_p);
         if (ps != PIDE2D_OK) return ps;
-        ps = run_precompute(H, mm, om_m, part, moment, par_m);
+        ps = run_precompute(H, mm, true, om_m, part, moment, par_m);
         if (ps != PIDE2D_OK) return ps;
         PIDE_CUDA(launch_central_difference(om_p, om_m, 0.5 / eps, reinterpret_cast<double*>(tb + t.dw + (size_t)k * t.omega),
                                             (size_t)N * N, s));
@@ -2294,7 +2295,7 @@ static pide2d_status price_create(pide2d_price* H, const pide2d_price_grid* g) {
     PIDE_PCUDA(launch_twiddles<double>(P, H->at<void>(H->off_twd), s));
     // weights on the z-lattice (N_z = nz, width hz), then conj(fft2(Omega padded))/P^2
     const int nzz = 2 * H->nz;
-    PIDE_PCUDA(precompute_core(nzz, H->hz, H->at<double>(H->off_gl), H->model, H->at<double>(H->off_omega),
+    PIDE_PCUDA(precompute_core(nzz, H->hz, H->at<double>(H->off_gl), H->model, false, H->at<double>(H->off_omega),
                                H->at<double>(H->off_part), H->at<double>(H->off_moment),
                                H->at<double>(H->off_params), s));
     PIDE_PCUDA(cudaMemcpy2DAsync(H->at<double>(H->off_pad), (size_t)(P / 2) * 8, H->at<double>(H->off_omega),

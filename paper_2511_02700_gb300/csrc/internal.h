@@ -374,13 +374,15 @@ constexpr int weights_rows(int N) { return N >= 2048 ? 4 : 1; }
 constexpr size_t weights_blocks(int N) {
     return (size_t)((N + 31) / 32) * ((N + 8 * weights_rows(N) - 1) / (8 * weights_rows(N)));
 }
-cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, double* omega, double* partials,
+// the same for the gradient's form (256 cells a block, in storage order)
+constexpr size_t gradient_weights_blocks(int N) { return ((size_t)N * N + 255) / 256; }
+cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, bool gradient, double* omega, double* partials,
                            int* nblocks, cudaStream_t s);
 // the R_I moment (eq. 3.3): blocks of the quadrature and the doubles of its buffer
 // (three moments, one spare, then the blocks' partial sums)
 constexpr int kMomentBlocks = 64;
 constexpr size_t moment_doubles() { return 4 + 3 * (size_t)kMomentBlocks; }
-cudaError_t launch_moment(const LevyParams& L, double H, const double* glx, const double* glw, int ngl,
+cudaError_t launch_moment(const LevyParams& L, bool gradient, double H, const double* glx, const double* glw, int ngl,
                           double tsh, double* out3, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int nblocks, const double* moment, double r,
                             const double* sigma_cov, double* params, cudaStream_t s);

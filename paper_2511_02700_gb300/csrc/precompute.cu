@@ -61,6 +61,42 @@ __device__ double log_ek(const LevyParams& L, double u) {
     return log(bessel_k_scaled(L.nu, exp(u)));
 }
 
+// The two forms of the density.  KEPT_POLY is the cheaper one: the interval's polynomial, one
+// logarithm for the table and for |z|^-nu.  LAGRANGE evaluates the interpolant from the table's
+// entries at ln(c1 |z|) and takes two.  They agree to rounding, but the gradient differences the
+// weights of models as little as 1e-8 apart in a drift, which multiplies the rounding of a weight,
+// and of the order in which weights are summed, by up to 1e8: for a drift near zero the two forms'
+// gradients differ by 1e-9 to 1e-8, about what either is off by.  The gradient's precomputes
+// therefore keep the one form, cell order and summation order it has always been computed with
+// (N = 256, 64 steps: 85.8 -> 87.5 ms for a gradient of twelve precomputes).
+enum class Density { KEPT_POLY, LAGRANGE };
+
+__device__ double log_ek_lagrange(const LevyParams& L, double x) {
+    if (L.ktab) {
+        const double f = (log(x) - L.ku0) * L.kidu;
+        const int base = (int)floor(f) - 3;
+        if (base >= 0 && base + 7 < L.kn) {
+            const double t = f - (double)base;             // in [3, 4)
+            // l_a(t) = prod_{b != a} (t - b) / (a - b) = pre_a suf_a c_a
+            constexpr double c[8] = {-1.0 / 5040.0, 1.0 / 720.0, -1.0 / 240.0, 1.0 / 144.0,
+                                     -1.0 / 144.0,  1.0 / 240.0, -1.0 / 720.0, 1.0 / 5040.0};
+            double pre[8], suf[8];
+            pre[0] = 1.0;
+#pragma unroll
+            for (int a = 1; a < 8; ++a) pre[a] = pre[a - 1] * (t - (double)(a - 1));
+            suf[7] = 1.0;
+#pragma unroll
+            for (int a = 6; a >= 0; --a) suf[a] = suf[a + 1] * (t - (double)(a + 1));
+            const double* T = L.ktab + base;
+            double v = 0.0;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) v += (pre[a] * suf[a] * c[a]) * T[a];
+            return v;
+        }
+    }
+    return log(bessel_k_scaled(L.nu, x));
+}
+
 // the interpolating polynomial of table entries i .. i + 7 in t, entry i + a at t = a - 7/2
 __global__ void k_kpoly(const double* __restrict__ tab, int n, double* __restrict__ poly) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -91,14 +127,20 @@ __global__ void k_kpoly(const double* __restrict__ tab, int n, double* __restric
 }
 
 // x^nu K_nu(x), bounded as x -> 0 (limit 2^(nu-1) Gamma(nu))
-__device__ double xnu_knu(const LevyParams& L, double x) {
+template <Density F> __device__ double xnu_knu(const LevyParams& L, double x) {
     if (x < 1e-8) return exp2(L.nu - 1.0) * L.gamma_nu;
+    if constexpr (F == Density::LAGRANGE) return exp(L.nu * log(x) - x + log_ek_lagrange(L, x));
     const double u = log(x);
     return exp(L.nu * u - x + log_ek(L, u));
 }
 
 // l(z), Sec. 4
-__device__ double levy_density(const LevyParams& L, double z1, double z2) {
+template <Density F> __device__ double levy_density(const LevyParams& L, double z1, double z2) {
+    if constexpr (F == Density::LAGRANGE) {
+        const double zn = sqrt(L.Ri11 * z1 * z1 + 2.0 * L.Ri12 * z1 * z2 + L.Ri22 * z2 * z2);
+        const double x = L.c1 * zn;
+        return exp(L.logpref + log_ek_lagrange(L, x) - x - L.nu * log(zn) + L.b1 * z1 + L.b2 * z2);
+    }
     // one logarithm serves K_nu's table and |z|^-nu
     const double q = L.Ri11 * z1 * z1 + 2.0 * L.Ri12 * z1 * z2 + L.Ri22 * z2 * z2;
     const double lz = 0.5 * log(q);
@@ -133,24 +175,26 @@ __global__ void k_ktab(double nu, double u0, double du, int n, double* tab) {
 // nodes in turn took longer than everything else (N = 128: 256 us for all
 // weights, 56 so; N = 1024 942 -> 567, N = 4096 13.2 -> 6.9 ms by the cheaper density).  Beyond, the cells are
 // numerous enough to fill the GPU one thread per cell, at full lane use.
-__host__ __device__ __forceinline__ int weights_warp_zone(const WeightJob& j) {
-    return j.M2 < 8 || j.N <= 256 ? j.M2 : 8;
+template <Density F> __host__ __device__ __forceinline__ int weights_warp_zone(const WeightJob& j) {
+    return j.M2 < 8 || (F == Density::KEPT_POLY && j.N <= 256) ? j.M2 : 8;
 }
 
 // the R_II cell integral at node (a, b) of its product rule (eq. 3.5 with the
 // |z|^2 factor of the modified midpoint rule)
+template <Density F>
 __device__ __forceinline__ double rii_node(const LevyParams& L, double c1, double c2, double h, const double* gx,
                                            const double* gw, int a, int b) {
     const double za = c1 + 0.5 * h * gx[a], zb = c2 + 0.5 * h * gx[b];
-    return gw[a] * gw[b] * (za * za + zb * zb) * levy_density(L, za, zb);
+    return gw[a] * gw[b] * (za * za + zb * zb) * levy_density<F>(L, za, zb);
 }
 
 // R_II cells with ||z_l||_inf / h in (2, weights_warp_zone]: one warp per cell of
 // the square around the origin, the rule's 100 nodes strided over the lanes
 // (at GB300's FP64 rate a cell's 100 density evaluations on one thread are the
 // tail of k_weights otherwise); the lane sums are added in a fixed order
+template <Density F>
 __global__ void k_weights_near(LevyParams L, WeightJob j, double* omega) {
-    const int Z = weights_warp_zone(j);
+    const int Z = weights_warp_zone<F>(j);
     const int side = 2 * Z;
     const int wcell = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -165,7 +209,7 @@ __global__ void k_weights_near(LevyParams L, WeightJob j, double* omega) {
     const double* gw = near ? j.gl_near_w : j.gl_far_w;
     const double c1 = (l1 + 0.5) * j.h, c2 = (l2 + 0.5) * j.h;
     double acc = 0.0;
-    for (int k = lane; k < n * n; k += 32) acc += rii_node(L, c1, c2, j.h, gx, gw, k / n, k - (k / n) * n);
+    for (int k = lane; k < n * n; k += 32) acc += rii_node<F>(L, c1, c2, j.h, gx, gw, k / n, k - (k / n) * n);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) {
@@ -178,17 +222,21 @@ __global__ void k_weights_near(LevyParams L, WeightJob j, double* omega) {
 // weights, eq. 3.5; one thread per cell, per-block partial sums of
 // (w, w (e^{z1} - 1), w (e^{z2} - 1)) for the deterministic final reduction
 // ---------------------------------------------------------------------------
+template <Density F>
 __global__ void k_weights(LevyParams L, WeightJob j, int rows, double* omega, double* partials) {
-    // 32 x 8 threads; a thread takes `rows` cells of its column, which share expm1(c1)
-    const int N = j.N;
-    const int i1 = blockIdx.x * 32 + threadIdx.x, lane = threadIdx.y * 32 + threadIdx.x;
+    // 32 x 8 threads; a thread takes `rows` cells of its column, which share expm1(c1), or, in the
+    // gradient's form, cell 256 blockIdx.x + lane of the rows one after another
+    constexpr bool FLAT = F == Density::LAGRANGE;
+    const int N = j.N, lane = threadIdx.y * 32 + threadIdx.x;
+    const int first = FLAT ? (int)blockIdx.x * 256 + lane : 0;
+    const int i1 = FLAT ? first % N : (int)(blockIdx.x * 32 + threadIdx.x);
     __shared__ double m2[32];
-    if (lane < 8 * rows) m2[lane] = expm1(((int)(blockIdx.y * 8 * rows) + lane - N / 2 + 0.5) * j.h);
+    if (!FLAT && lane < 8 * rows) m2[lane] = expm1(((int)(blockIdx.y * 8 * rows) + lane - N / 2 + 0.5) * j.h);
     __syncthreads();
     const double m1 = expm1((i1 - N / 2 + 0.5) * j.h);
     double w0 = 0.0, e1 = 0.0, e2 = 0.0;
     for (int r = 0; r < rows; ++r) {
-        const int row = threadIdx.y + 8 * r, i2 = blockIdx.y * 8 * rows + row;
+        const int row = threadIdx.y + 8 * r, i2 = FLAT ? first / N : (int)(blockIdx.y * 8 * rows + row);
         if (i1 >= N || i2 >= N) break;
         const size_t cell = (size_t)i2 * N + i1;
         double w = 0.0;
@@ -197,7 +245,7 @@ __global__ void k_weights(LevyParams L, WeightJob j, int rows, double* omega, do
         const double inf = fmax(fabs(l1 + 0.5), fabs(l2 + 0.5));   // ||z_l||_inf / h
         if (inf <= 2.0) {
             w = 0.0;                                               // R_I
-        } else if (inf <= (double)weights_warp_zone(j)) {
+        } else if (inf <= (double)weights_warp_zone<F>(j)) {
             w = omega[cell];                                       // R_II near the origin: k_weights_near
         } else if (inf <= (double)j.M2) {                          // R_II
             // Gauss-Legendre order by distance from the singular origin (in
@@ -214,18 +262,18 @@ __global__ void k_weights(LevyParams L, WeightJob j, int rows, double* omega, do
                 double inner = 0.0;
                 for (int b = 0; b < n; ++b) {
                     const double zb = c2 + 0.5 * j.h * gx[b];
-                    inner += gw[b] * (za * za + zb * zb) * levy_density(L, za, zb);
+                    inner += gw[b] * (za * za + zb * zb) * levy_density<F>(L, za, zb);
                 }
                 acc += gw[a] * inner;
             }
             w = acc * 0.25 * j.h * j.h / (c1 * c1 + c2 * c2);
         } else {                                                   // R_III
-            w = levy_density(L, c1, c2) * j.h * j.h;
+            w = levy_density<F>(L, c1, c2) * j.h * j.h;
         }
         omega[cell] = w;
         w0 += w;
         e1 += w * m1;
-        e2 += w * m2[row];
+        e2 += w * (FLAT ? expm1(c2) : m2[row]);
     }
     __shared__ double sw[256], s1[256], s2[256];
     sw[lane] = w0;
@@ -253,6 +301,7 @@ __global__ void k_weights(LevyParams L, WeightJob j, int rows, double* omega, do
 // ---------------------------------------------------------------------------
 // kMomentBlocks blocks each sum a strided share of the nodes into part[3 b ..];
 // k_moment_sum adds the partial sums in block order (deterministic)
+template <Density F>
 __global__ void k_moment(LevyParams L, double H, const double* glx, const double* glw, int ngl, double tsh,
                          double* part) {
     const double pi = 3.141592653589793;
@@ -281,9 +330,9 @@ __global__ void k_moment(LevyParams L, double H, const double* glx, const double
         else { d1 = t; d2 = -1.0; }
         const double dn = sqrt(L.Ri11 * d1 * d1 + 2.0 * L.Ri12 * d1 * d2 + L.Ri22 * d2 * d2);
         const double ed = L.b1 * d1 + L.b2 * d2;
-        // rho^3 d d^T l(rho d) = rho^(1-2 alpha) d d^T F, F = rho^(2 nu) l(rho d)
-        const double F = L.pref0 * xnu_knu(L, L.c1 * dn * rho) * pow(dn, -2.0 * L.nu) * exp(rho * ed);
-        const double g = wr * glw[ti] * pow(rho, 1.0 - 2.0 * L.alpha) * F;
+        // rho^3 d d^T l(rho d) = rho^(1-2 alpha) d d^T G, G = rho^(2 nu) l(rho d)
+        const double G = L.pref0 * xnu_knu<F>(L, L.c1 * dn * rho) * pow(dn, -2.0 * L.nu) * exp(rho * ed);
+        const double g = wr * glw[ti] * pow(rho, 1.0 - 2.0 * L.alpha) * G;
         m11 += g * d1 * d1;
         m12 += g * d1 * d2;
         m22 += g * d2 * d2;
@@ -515,24 +564,33 @@ __global__ void k_ring(Geometry g, const double* E1d, const double* E2d, double 
 }
 
 // ---------------------------------------------------------------------------
-cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, double* omega, double* partials, int* nblocks,
-                           cudaStream_t s) {
-    // four rows a thread save exponentials and partial sums where the cells fill the chip
-    const int rows = weights_rows(j.N);
-    *nblocks = (int)weights_blocks(j.N);
-    const dim3 grd((j.N + 31) / 32, *nblocks / ((j.N + 31) / 32));
-    const int side = 2 * weights_warp_zone(j);
-    k_weights_near<<<(side * side + 7) / 8, 256, 0, s>>>(L, j, omega);       // eight cells per block
+template <Density F>
+static cudaError_t launch_weights_form(const LevyParams& L, const WeightJob& j, dim3 grd, int rows, double* omega,
+                                       double* partials, cudaStream_t s) {
+    const int side = 2 * weights_warp_zone<F>(j);
+    k_weights_near<F><<<(side * side + 7) / 8, 256, 0, s>>>(L, j, omega);       // eight cells per block
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_weights<<<grd, dim3(32, 8), 0, s>>>(L, j, rows, omega, partials);
+    k_weights<F><<<grd, dim3(32, 8), 0, s>>>(L, j, rows, omega, partials);
     return cudaGetLastError();
 }
-cudaError_t launch_moment(const LevyParams& L, double H, const double* glx, const double* glw, int ngl, double tsh,
-                          double* out3, cudaStream_t s) {
+cudaError_t launch_weights(const LevyParams& L, const WeightJob& j, bool gradient, double* omega, double* partials,
+                           int* nblocks, cudaStream_t s) {
+    if (gradient) {
+        *nblocks = (int)gradient_weights_blocks(j.N);
+        return launch_weights_form<Density::LAGRANGE>(L, j, dim3(*nblocks), 1, omega, partials, s);
+    }
+    // four rows a thread save exponentials and partial sums where the cells fill the chip
+    *nblocks = (int)weights_blocks(j.N);
+    const dim3 grd((j.N + 31) / 32, *nblocks / ((j.N + 31) / 32));
+    return launch_weights_form<Density::KEPT_POLY>(L, j, grd, weights_rows(j.N), omega, partials, s);
+}
+cudaError_t launch_moment(const LevyParams& L, bool gradient, double H, const double* glx, const double* glw, int ngl,
+                          double tsh, double* out3, cudaStream_t s) {
     // out3 holds the three moments, then kMomentBlocks x 3 partial sums (moment_doubles())
     double* part = out3 + 4;
-    k_moment<<<kMomentBlocks, 256, 0, s>>>(L, H, glx, glw, ngl, tsh, part);
+    if (gradient) k_moment<Density::LAGRANGE><<<kMomentBlocks, 256, 0, s>>>(L, H, glx, glw, ngl, tsh, part);
+    else k_moment<Density::KEPT_POLY><<<kMomentBlocks, 256, 0, s>>>(L, H, glx, glw, ngl, tsh, part);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_moment_sum<<<1, 32, 0, s>>>(part, kMomentBlocks, out3);
@@ -546,7 +604,7 @@ cudaError_t launch_finalize(const double* partials, int nblocks, const double* m
 cudaError_t launch_ktab(double nu, double u0, double du, int n, double* tab, double* poly, cudaStream_t s) {
     k_ktab<<<(n + 3) / 4, 128, 0, s>>>(nu, u0, du, n, tab);      // four entries per block
     const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !poly) return e;
     k_kpoly<<<(n + 127) / 128, 128, 0, s>>>(tab, n, poly);
     return cudaGetLastError();
 }
