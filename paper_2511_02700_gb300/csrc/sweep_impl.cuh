@@ -105,8 +105,10 @@ __device__ __forceinline__ R diff_state(const S* Y, size_t idx, int ld, R d11, R
 // division (2 ulp; max(1, |y|) stays far below 2^126), since the selected node is evaluated
 // again in FP64.  In FP64 ratios are compared by products, three FP64 instructions a node
 // instead of about twenty with a quotient (two FP64 lanes per SM), and one quotient is
-// formed at the end; max(1, |y|) and the test for NaN run on the integer pipe.  A NaN
-// ratio or y marks the block non-finite.
+// formed at the end; max(1, |y|) and the test of the exponents run on the integer pipe.  The
+// products of values from 2^511 on could overflow: from the first such value on, a thread
+// compares quotients.  A NaN or infinite increment or y marks the block non-finite (in FP32, as a
+// NaN ratio: an infinite increment makes y infinite).
 template <typename R> struct StopSel;
 template <> struct StopSel<float> {
     float q = -1.f, d = 0.f;
@@ -122,15 +124,13 @@ template <> struct StopSel<float> {
 };
 template <> struct StopSel<double> {
     double d = -1.0, m = 1.0, y = 0.0;       // |d| of the selected node (-1: none), max(1, |y|), y
-    bool bad = false;
-    static __device__ __forceinline__ bool is_nan(double x) {
-        return (unsigned)(__double2hiint(x) & 0x7fffffff) + (__double2loint(x) != 0 ? 1u : 0u) > 0x7ff00000u;
-    }
+    bool bad = false, wide = false;
     __device__ __forceinline__ void add(double dn, double yn) {
-        const double a = fabs(dn);
-        const double mn = (__double2hiint(yn) & 0x7fffffff) < 0x3ff00000 ? 1.0 : fabs(yn);
-        bad |= is_nan(dn) || is_nan(yn);
-        if (a * m > d * mn) { d = a; m = mn; y = yn; }
+        const int hd = __double2hiint(dn) & 0x7fffffff, hy = __double2hiint(yn) & 0x7fffffff;
+        const double a = fabs(dn), mn = hy < 0x3ff00000 ? 1.0 : fabs(yn);
+        wide |= max(hd, hy) >= 0x5fe00000;
+        bad |= max(hd, hy) >= 0x7ff00000;
+        if (wide ? a / mn > ratio() : a * m > d * mn) { d = a; m = mn; y = yn; }
     }
     __device__ __forceinline__ double ratio() const { return d < 0.0 ? -1.0 : d / m; }
 };
