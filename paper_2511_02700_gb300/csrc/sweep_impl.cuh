@@ -1017,7 +1017,8 @@ __device__ __forceinline__ void col_solve_f64(const ColSolveArgs<double>& a, int
         // lane: column lane & 1, powers r = lane / 2 + 1
         const int cl = threadIdx.x & 1, r = (threadIdx.x >> 1) + 1;
         const R sv = (a.rc0 + a.rc1 * a.sin2[ka + cl]) / cc;
-        const R w = R(0.5) * sv + sqrt(sv + R(0.25) * sv * sv);
+        // (w = s to rounding where s^2 would overflow: time steps of less than 1e-150)
+        const R w = sv < R(1e100) ? R(0.5) * sv + sqrt(sv + R(0.25) * sv * sv) : sv;
         const R q = R(1) / (R(1) + w);
         PsiPow x{R(0), R(1)}, y{w * q * (R(1) + q), q * q};
         R pw = R(1), yw = q;
