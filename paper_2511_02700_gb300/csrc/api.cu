@@ -1186,10 +1186,11 @@ static pide2d_status do_create(pide2d* H) {
 
 // whether kernels may read or write a caller's array of doubles in place: memory of the
 // current device, aligned to its elements.  Anything else (host, managed, another device)
-// is staged in R_OUT by a strided copy.  In place, the odd pitch of (N+1) doubles costs the
-// kernels little, where a strided copy each way and a conversion between pitches cost more
-// than an iteration's passes: N = 4096 FP32-bulk probe 1.62 -> 1.21 ms, N = 512 jump sum 87 -> 70 us.
-static bool direct_field(const double* p) {
+// is staged by a strided copy (in R_OUT; pide2d_jump_static in its own scratch).  In place, the
+// odd pitch of (N+1) doubles costs the kernels little, where a strided copy each way and a
+// conversion between pitches cost more than an iteration's passes: N = 4096 FP32-bulk probe
+// 1.62 -> 1.21 ms, N = 512 jump sum 87 -> 70 us.
+bool pide::direct_field(const double* p) {
     if (((uintptr_t)p & 7) != 0) return false;
     cudaPointerAttributes at{};
     int dev = -1;

@@ -202,6 +202,7 @@ template <typename R> cudaError_t launch_dst_row_jobs(const DstRowArgs<R>& a0, c
                                                      JobsCtl jc, int upb, cudaStream_t s);
 // the single-job units per block of the FFT kernels at transform length P (0 if P is unsupported)
 int fft_units_per_block(int P, int prec_bytes);
+bool direct_field(const double* p);     // a caller's array that kernels take in place (api.cu)
 template <typename R> cudaError_t launch_prep_jobs(const PrepArgs<R>& a0, const PrepArgs<R>* arr, int K,
                                                   bool explicit_part, cudaStream_t s);
 // price-space jump operator (eqs. 3.12-3.17 on the paper's price grid); P x P transforms

@@ -135,9 +135,10 @@ extern "C" pide2d_status pide2d_jump_static(int n, const double* omega, const do
     PIDE_STATIC_CUDA(launch_row_forward<double>(wa, s));
     PIDE_STATIC_CUDA(launch_weights_col<double>(gd, Wt, Wh, nullptr, tw, s));
 
-    // one zero-padded correlation sweep of U, read in place (staged when it is not aligned
-    // to its elements)
-    const bool in_place = ((uintptr_t)U & 7) == 0, out_place = ((uintptr_t)out & 7) == 0;
+    // one zero-padded correlation sweep of U, read in place where it is memory of this device
+    // aligned to its elements, else staged by a copy, which moves what kernels cannot reach or
+    // returns a status
+    const bool in_place = direct_field(U), out_place = direct_field(out);
     if (!in_place)
         PIDE_STATIC_CUDA(cudaMemcpy2DAsync(X, (size_t)g.ldS * 8, U, (size_t)(n + 1) * 8, (size_t)(n + 1) * 8, n + 1,
                                            cudaMemcpyDeviceToDevice, s));
