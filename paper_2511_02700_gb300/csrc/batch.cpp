@@ -30,8 +30,20 @@ void set_global_error(const std::string& msg);
 size_t group_scratch_bytes(int K, int n_steps);
 pide2d_status solve_group(pide2d_t* const* hs, int K, void* scratch, int upb, std::string* err);
 pide2d_status time_col_jobs(pide2d_t* const* hs, int K, void* scratch, int upb, int reps, double* ms, std::string* err);
-int fft_units_per_block(int P, int prec_bytes);
+struct FftShape {
+    int units, unit_threads, max_threads;
+};
+FftShape fft_shape(int P, int prec_bytes);
+int batch_trial_units(int N, int prec, int* units);
 void set_handle_stream(pide2d_t* h, void* stream);
+}
+
+// units per block of the trials (at most three), ascending
+int pide::batch_trial_units(int N, int prec, int* units) {
+    const FftShape f = fft_shape(2 * N, prec == PIDE2D_FP64 ? 8 : 4);
+    int n = 0;
+    for (int u = f.units; n < 3 && u * f.unit_threads <= f.max_threads; u *= 2) units[n++] = u;
+    return n;
 }
 
 namespace {
@@ -42,23 +54,23 @@ constexpr int kTrialReps = 3;
 // Launch shape of a geometry group, picked by timed trials on its first
 // chunk (the column pass of the fixed-point iteration, the heaviest multi-job
 // kernel): FFT units per block among 1x, 2x, 4x the single-job shape (up to
-// 512 threads), then jobs per chunk among the chunk size and its half (a
-// smaller chunk wins only if its time per job is 3% lower).
+// the kernels' most threads, each shape once), then jobs per chunk among the chunk size and its
+// half (a smaller chunk wins only if its time per job is 3% lower).  Blocks of more units have
+// been the slower ones since units hold 4 or 8 values a thread; the time loops of 48 jobs with
+// 1, 2, 4 units: N = 128 FP32 13.8, 13.7, 14.3 ms, FP64 39.7, 40.2, 44.2 ms; N = 256 FP32 55.2, 55.1,
+// 57.6 ms, FP64 234, 256, 318 ms.
 struct Shape {
     int upb = 0, lanes = 0;
     double us_per_job = 0.0;
 };
 
 pide2d_status tune_shape(pide2d_t* const* hs, int K, void* scratch, int N, int prec, Shape* out, std::string* err) {
-    const int base = pide::fft_units_per_block(2 * N, prec == PIDE2D_FP64 ? 8 : 4);
-    const int nt = (2 * N) / 16;
     Shape best;
     double best_ms = 1e300;
-    int last = -1;
-    for (int f : {1, 2, 4}) {
-        const int u = std::min(base * f, std::max(1, 512 / nt));
-        if (u == last) continue;
-        last = u;
+    int units[3];
+    const int n = pide::batch_trial_units(N, prec, units);
+    for (int i = 0; i < n; ++i) {
+        const int u = units[i];
         double ms = 0.0;
         const pide2d_status st = pide::time_col_jobs(hs, K, scratch, u, kTrialReps, &ms, err);
         if (st != PIDE2D_OK) return st;

@@ -201,7 +201,12 @@ template <typename R> cudaError_t launch_col_solve_jobs(const ColSolveArgs<R>& a
 template <typename R> cudaError_t launch_dst_row_jobs(const DstRowArgs<R>& a0, const DstRowArgs<R>* arr, int K,
                                                      JobsCtl jc, int upb, cudaStream_t s);
 // the single-job units per block of the FFT kernels at transform length P (0 if P is unsupported)
-int fft_units_per_block(int P, int prec_bytes);
+// launch shape of the FFT kernels of length P: units per block of a single solve, threads per
+// unit, and the most threads per block of the multi-job kernels
+struct FftShape {
+    int units, unit_threads, max_threads;
+};
+FftShape fft_shape(int P, int prec_bytes);
 bool direct_field(const double* p);     // a caller's array that kernels take in place (api.cu)
 template <typename R> cudaError_t launch_prep_jobs(const PrepArgs<R>& a0, const PrepArgs<R>* arr, int K,
                                                   bool explicit_part, cudaStream_t s);

@@ -36,13 +36,15 @@ PIDE_INSTANTIATE(PIDE_PREC)
 }  // namespace pide
 
 namespace pide {
-int fft_units_per_block(int P, int prec_bytes) {
-#define CASE(PP) return prec_bytes == 4 ? Cfg<float, PP>::UNITS : Cfg<double, PP>::UNITS;
+FftShape fft_shape(int P, int prec_bytes) {
+#define CASE(PP)                                                                                     \
+    return prec_bytes == 4 ? FftShape{Cfg<float, PP>::UNITS, Cfg<float, PP>::NT, Cfg<float, PP>::MAXT} \
+                           : FftShape{Cfg<double, PP>::UNITS, Cfg<double, PP>::NT, Cfg<double, PP>::MAXT};
     switch (P) {
         case 16: CASE(16); case 32: CASE(32); case 64: CASE(64); case 128: CASE(128);
         case 256: CASE(256); case 512: CASE(512); case 1024: CASE(1024);
         case 2048: CASE(2048); case 4096: CASE(4096); case 8192: CASE(8192);
-        default: return 0;
+        default: return FftShape{0, 0, 0};
     }
 #undef CASE
 }

@@ -53,7 +53,8 @@ template <typename R, int P> struct Cfg {
     static constexpr int MINB = TPS / THREADS < 24 ? TPS / THREADS : 24;
     static constexpr size_t SMEM = (size_t)UNITS * ULEN * sizeof(cpx<R>);
     // multi-job kernels: launched with any number of units per block up to
-    // MAXT threads (the batch picks it by timed trials), same register target
+    // MAXT threads (the batch picks it by timed trials); 64 registers a thread in FP32, 128 in
+    // FP64, there also at P = 2048 and 4096
     static constexpr int MAXT = THREADS > 512 ? THREADS : 512;
     static constexpr int JMINB = (sizeof(R) == 4 ? 1024 : 512) / MAXT > 0 ? (sizeof(R) == 4 ? 1024 : 512) / MAXT : 1;
 };
