@@ -106,9 +106,10 @@ __device__ __forceinline__ R diff_state(const S* Y, size_t idx, int ld, R d11, R
 // division (2 ulp; max(1, |y|) stays far below 2^126), since the selected node is evaluated
 // again in FP64.  In FP64 ratios are compared by products, three FP64 instructions a node
 // instead of about twenty with a quotient (two FP64 lanes per SM), and one quotient is
-// formed at the end; max(1, |y|) and the test of the exponents run on the integer pipe.  The
-// products of values from 2^511 on could overflow: from the first such value on, a thread
-// compares quotients.  A NaN or infinite increment or y marks the block non-finite (in FP32, as a
+// formed at the end; max(1, |y|) and the largest exponent run on the integer pipe.  Products of
+// values from 2^511 on could overflow: a thread that met one selects again by quotients from the
+// stored D and Y (quotients in the loop: 48 jobs of N = 256 229 -> 233 ms; scaled products: N = 512 solve
+// 54.0 -> 55.5 ms).  A NaN or infinite increment or y marks the block non-finite (in FP32, as a
 // NaN ratio: an infinite increment makes y infinite).
 template <typename R> struct StopSel;
 template <> struct StopSel<float> {
@@ -121,18 +122,24 @@ template <> struct StopSel<float> {
         bad |= !(r == r) || !(yr == yr);
         if (r > q) { q = r; d = dn; y = yn; }
     }
+    __device__ __forceinline__ bool non_finite() const { return bad; }
     __device__ __forceinline__ float ratio() const { return q; }
 };
 template <> struct StopSel<double> {
     double d = -1.0, m = 1.0, y = 0.0;       // |d| of the selected node (-1: none), max(1, |y|), y
-    bool bad = false, wide = false;
+    int top = 0;                             // largest high word of |d| and |y|
     __device__ __forceinline__ void add(double dn, double yn) {
-        const int hd = __double2hiint(dn) & 0x7fffffff, hy = __double2hiint(yn) & 0x7fffffff;
+        const int hy = __double2hiint(yn) & 0x7fffffff;
         const double a = fabs(dn), mn = hy < 0x3ff00000 ? 1.0 : fabs(yn);
-        wide |= max(hd, hy) >= 0x5fe00000;
-        bad |= max(hd, hy) >= 0x7ff00000;
-        if (wide ? a / mn > ratio() : a * m > d * mn) { d = a; m = mn; y = yn; }
+        top = max(top, max(__double2hiint(dn) & 0x7fffffff, hy));
+        if (a * m > d * mn) { d = a; m = mn; y = yn; }
     }
+    __device__ __forceinline__ void add_large(double dn, double yn) {
+        const double a = fabs(dn), mn = fmax(1.0, fabs(yn));
+        if (a / mn > ratio()) { d = a; m = mn; y = yn; }
+    }
+    __device__ __forceinline__ bool large() const { return top >= 0x5fe00000 && top < 0x7ff00000; }
+    __device__ __forceinline__ bool non_finite() const { return top >= 0x7ff00000; }
     __device__ __forceinline__ double ratio() const { return d < 0.0 ? -1.0 : d / m; }
 };
 
@@ -1303,6 +1310,17 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
 #pragma unroll
             for (int i = 0; i < EB; ++i) update(t + NT * (b0 + i), zz[b0 + i], y0[i], y1[i]);
         }
+        if constexpr (sizeof(R) == 8) {
+            if (sel.large()) {
+                sel.d = -1.0;
+#pragma unroll 1
+                for (int m1 = t; m1 < N; m1 += NT) {
+                    if (m1 < 1) continue;
+                    sel.add_large(a.D[(size_t)m2 * ldR + m1], Yv[(size_t)m2 * ld + m1]);
+                    if (hasb) sel.add_large(a.D[(size_t)(m2 + 1) * ldR + m1], Yv[(size_t)(m2 + 1) * ld + m1]);
+                }
+            }
+        }
         __syncthreads();
     }
     // (reduced here, before the second transform, so the candidate's registers
@@ -1314,7 +1332,7 @@ __device__ __forceinline__ void dst_row_body(const DstRowArgs<R>& a, int upb) {
     // is within 2^-20 relative of the exact FP64 maximum.
     R qmax = sel.ratio(), dsel = sel.d;
     St<R> ysel = sel.y;
-    bool bad = sel.bad;
+    bool bad = sel.non_finite();
     for (int o = 16; o > 0; o >>= 1) {
         const R oq = __shfl_xor_sync(0xffffffffu, qmax, o);
         const R od = __shfl_xor_sync(0xffffffffu, dsel, o);
