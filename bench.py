@@ -639,7 +639,7 @@ def run_paper_schemes(B, torch, dev):
             price = _bilinear_at(x, V, ps.strike, ps.strike)
             res["price_space"].append({
                 "set": name, "n_x": nx, "precision": prec, "time_steps": nx // 2, "status": status, "wall_s": wall,
-                "fp_iters_total": st.fp_iters_total, "cell_iterations_per_s": st.cell_iters / wall,
+                "fp_iters_total": st.fp_iters_total, "fp_iterations_per_s": st.fp_iters_total / wall,
                 "price_at_KK": price, "table4_at_KK": ps.table4_at_k, "diff": price - ps.table4_at_k})
     ps = PAPER_SETS["VG0"]
     n, hw = 2048, 11.5

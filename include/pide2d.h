@@ -121,7 +121,9 @@ typedef struct {
     int fp_iters_max;     /* largest per-step count                               */
     double last_resid;    /* last eq. 3.25 quantity of the last step              */
     double cell_iters;    /* N^2 * (fixed-point iterations + 1) summed: the number */
-                          /* of grid-cell applications of B_w                     */
+                          /* of grid-cell applications of B_w (nominal in         */
+                          /* pide2d_price_solve: FP64 forms one of them from kept */
+                          /* ones)                                                */
 } pide2d_stats;
 
 typedef struct pide2d pide2d_t;

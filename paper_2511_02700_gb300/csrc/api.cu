@@ -2556,7 +2556,7 @@ static pide2d_status price_solve(pide2d_price* H, const pide2d_contract* c, doub
         pide2d_status js = apply_jump(fld(out_field), fld(bv(out_field)));
         if (js != PIDE2D_OK) return js;
         S.fp_iters_total += k;
-        S.cell_iters += (double)n * (k + 1);
+        S.cell_iters += (double)n * (k + 1);       // (with by_ready the start's is a combination of kept ones)
         return PIDE2D_OK;
     };
     int first = 1;

@@ -228,6 +228,9 @@ __device__ __forceinline__ void dft_small(C* v) {
 //   FP32  P = 256 37.7 -> 26.1 us (4 values; 8 take 29.4), P = 512 40.1 -> 31.8 us (8).
 //         P = 1024: 45.7 -> 42.3 us with 8 for one solve, but a batch of 44
 //         N = 512 jobs goes from 326 to 383 ms, so 16 stay from there on.
+// The multi-job kernels take the same choice, since a batch returns the bits of single solves.
+// Their FP32 time loops, 16 values against it: 16 jobs of N = 128 9.2 -> 7.0 ms, of N = 256 24.3 -> 23.2;
+// 48 jobs, which fill the chip, of N = 64 6.2 -> 4.8, of N = 128 13.0 -> 13.7, of N = 256 53.2 -> 55.1.
 template <typename R> __host__ __device__ constexpr int fft_values(int P) {
     if (sizeof(R) == 8) return P <= 512 ? 4 : (P <= 4096 ? 8 : 16);
     return P <= 256 ? 4 : (P <= 512 ? 8 : 16);
