@@ -10,7 +10,11 @@
 // at 2^-58 of its largest value; an FP64 butterfly rounds every value at 2^-53 of
 // itself.  Against long double, over noise, payoff-like, decaying and peaked sequences of
 // 128 to 8192 values, the error is half that of a radix-2 FP64 transform (equal for a
-// single spike at 8192).
+// single spike at 8192).  A spectrum column keeps its entries to 2^-61 of its largest and the
+// product its values to 2^-62 of the two maxima's, below the transforms' own errors: jump
+// sums with spectra that fall by 1e-8 within a column, or peak where the field's do not, are
+// off by 0.04 to 0.51 of what they were with FP64 butterflies (N = 64 to 256, against 128 bits).
+// Subnormal values count as zero, so fields below about 1e-288 lose digits.
 //
 // Measured, one fixed-point iteration of a solve with FP64 transforms against these:
 // N = 256 75 -> 56 us, N = 512 213 -> 113 us, N = 1024 755 -> 339 us (column pass 297 -> 90,
